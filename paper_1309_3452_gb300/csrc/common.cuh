@@ -86,9 +86,10 @@ struct F32 {
 // A plane-wave link factor exp(-i phi) = c - i s of the FP32 kernels' per-step
 // table (c = c_hi + c_lo, s = s_hi + s_lo), kept as the packed operand pairs
 // of plane_link_diff: ch = (c_hi, c_hi), cl = (c_lo, c_lo), sh = (s_hi, -s_hi),
-// sl = (s_lo, -s_lo)
+// sl = (s_lo, -s_lo) (one value: lanes re, im) and sp = (s_hi, s_hi), lp =
+// (s_lo, s_lo) (two values: lanes are the two sublattices, quad.cuh)
 struct PlaneLink32 {
-  float2 ch, cl, sh, sl;
+  float2 ch, cl, sh, sl, sp, lp;
 };
 
 __device__ __forceinline__ double2 cmk(double a, double b) { return make_double2(a, b); }
@@ -585,7 +586,35 @@ struct HalfFields {
   // neighbour (applied conjugated, like the per-site path)
   const typename P::Link* larr;
   long long larr_n, larr_ps;
+  // the two tables of a simulation whose state is held as sublattice quads
+  // (quad.cuh; F32 only, then b_tab and larr are null): per component cell
+  // two float4, {re hi 0, re hi 1, im hi 0, im hi 1} and the lo parts, at
+  // 2 (component * q_ps + site), the link table's slots (2 axis + dir) one
+  // after another
+  const float4* bq;
+  const float4* lq;
+  long long q_ps;
 };
+
+// one value's {re hi, im hi, re lo, im lo} from a quad record
+__device__ __forceinline__ float4 quad_lane(const float4* rec, int lane) {
+  const float4 h = __ldg(rec), l = __ldg(rec + 1);
+  return lane ? make_float4(h.y, h.w, l.y, l.w) : make_float4(h.x, h.z, l.x, l.z);
+}
+// LINK_TABLE: a value's link factor of one slot
+template <int DIMS>
+__device__ __forceinline__ F64::Link table_link(const HalfFields<F64>& h, int slot, int plane, long long site) {
+  return h.larr[slot * h.larr_n + (long long)plane * h.larr_ps + site];
+}
+template <int DIMS>
+__device__ __forceinline__ F32::Link table_link(const HalfFields<F32>& h, int slot, int plane, long long site) {
+  if (h.lq) {
+    const long long i = (long long)(slot * (nplanes<DIMS>() / 2) + (plane >> 1)) * h.q_ps + site;
+    const float4 v = quad_lane(h.lq + 2 * i, plane & 1);
+    return F32::Link{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+  }
+  return h.larr[slot * h.larr_n + (long long)plane * h.larr_ps + site];
+}
 
 // The tabulated-potential update (F32 only), the paper's form of the Cayley
 // step (Eqs. ss1-ss4):  F+ = b (2F - S) - F,  b = 1/(1 + i theta),  S = r_x S'
@@ -603,7 +632,8 @@ __device__ __forceinline__ double2 apply_table<F64>(const HalfFields<F64>&, doub
 template <>
 __device__ __forceinline__ float2 apply_table<F32>(const HalfFields<F32>& h, float2 F, float2 S, int plane,
                                                    long long site) {
-  const float4 b = __ldg(h.b_tab[plane] + site);
+  const float4 b = h.bq ? quad_lane(h.bq + 2 * ((plane >> 1) * h.q_ps + site), plane & 1)
+                        : __ldg(h.b_tab[plane] + site);
   // w = 2F - r_x S'  (small product first)
   const float2 w = pfma(make_float2(-h.rx_hi, -h.rx_hi), S,
                         pfma(make_float2(-h.rx_lo, -h.rx_lo), S, padd(F, F)));
@@ -669,65 +699,31 @@ __device__ __forceinline__ long long softcore_corr_index(int plane, const int (&
   return ((long long)yr * N[0] + x) * 4 + plane;
 }
 
-// COEF_SOFTCORE update (FP32 only): b of this value from the caller's pair
-// computation (bpre) or computed here (both lanes the same value, so the
-// result is bit-identical to the value's lane of a pair)
+// COEF_SOFTCORE update (FP32 only): b of this value (both lanes the same value,
+// so the result is bit-identical to the value's lane of a pair)
 template <int DIMS, class P>
 __device__ __forceinline__ typename P::cplx apply_softcore(const HalfFields<P>& h, typename P::cplx F,
-                                                           typename P::cplx S, const int (&H)[3],
-                                                           const float4* bpre);
-template <>
-__device__ __forceinline__ double2 apply_softcore<2, F64>(const HalfFields<F64>&, double2 F, double2,
-                                                          const int (&)[3], const float4*) {
-  return F;  // not used: FP64 kernels take the general path
-}
-template <>
-__device__ __forceinline__ double2 apply_softcore<3, F64>(const HalfFields<F64>&, double2 F, double2,
-                                                          const int (&)[3], const float4*) {
-  return F;
-}
-template <int DIMS>
-__device__ __forceinline__ float2 apply_softcore_f32(const HalfFields<F32>& h, float2 F, float2 S,
-                                                     const int (&H)[3], const float4* bpre) {
-  float4 b;
-  if (bpre) {
-    b = *bpre;
-  } else {
+                                                           typename P::cplx S, const int (&H)[3]) {
+  if constexpr (sizeof(typename P::real) == 4) {
     float Rh, Rl;
     softcore_R<DIMS>(h, H, Rh, Rl);
     const float2 t0 = softcore_t0(h, H);
-    b = lane_b(softcore_b2(f2(Rh), f2(Rl), f2(t0.x), f2(t0.y), h.sc_K_hi, h.sc_K_lo), 0);
+    const float4 b = lane_b(softcore_b2(f2(Rh), f2(Rl), f2(t0.x), f2(t0.y), h.sc_K_hi, h.sc_K_lo), 0);
+    return apply_b(b, h.rx_hi, h.rx_lo, F, S);
+  } else {
+    return F;  // not used: FP64 kernels take the general path
   }
-  return apply_b(b, h.rx_hi, h.rx_lo, F, S);
 }
 // COEF_SOFTCORR: the FP32 estimate of this value plus its tabulated correction
-// (or the caller's pair computation, bpre)
 template <int DIMS>
 __device__ __forceinline__ float2 apply_softcorr_f32(const HalfFields<F32>& h, float2 F, float2 S,
-                                                     const int (&H)[3], const float4* bpre, int plane,
-                                                     const int (&N)[3]) {
-  float4 b;
-  if (bpre) {
-    b = *bpre;
-  } else {
-    float Rh, Rl;
-    softcore_R<DIMS>(h, H, Rh, Rl);
-    float2 re, im;
-    softcore_fast2(f2(Rh), f2(Rl), f2(softcore_t0(h, H).x), h.sc_K_hi, re, im);
-    const float2 c = corr_decode(__ldg(h.sc_corr + softcore_corr_index<DIMS>(plane, H, N)));
-    b = make_float4(re.x, c.x, im.x, c.y);
-  }
-  return apply_b(b, h.rx_hi, h.rx_lo, F, S);
-}
-template <>
-__device__ __forceinline__ float2 apply_softcore<2, F32>(const HalfFields<F32>& h, float2 F, float2 S,
-                                                         const int (&H)[3], const float4* bpre) {
-  return apply_softcore_f32<2>(h, F, S, H, bpre);
-}
-template <>
-__device__ __forceinline__ float2 apply_softcore<3, F32>(const HalfFields<F32>& h, float2 F, float2 S,
-                                                         const int (&H)[3], const float4* bpre) {
-  return apply_softcore_f32<3>(h, F, S, H, bpre);
+                                                     const int (&H)[3], int plane, const int (&N)[3]) {
+  float Rh, Rl;
+  softcore_R<DIMS>(h, H, Rh, Rl);
+  float2 re, im;
+  softcore_fast2(f2(Rh), f2(Rl), f2(softcore_t0(h, H).x), h.sc_K_hi, re, im);
+  const float2 c = corr_decode(__ldg(h.sc_corr + softcore_corr_index<DIMS>(plane, H, N)));
+  return apply_b(make_float4(re.x, c.x, im.x, c.y), h.rx_hi, h.rx_lo, F, S);
 }
 
 // Field-path selectors for site_update: a fixed CoefMode / LinkMode compiles
@@ -746,7 +742,6 @@ __device__ __forceinline__ typename P::cplx site_update(
     const HalfFields<P>& h, const FieldDesc& f, bool iso, const typename P::Ratio& ry,
     const typename P::Ratio& rz, int plane, typename P::cplx F, typename P::cplx (&nb)[6],
     const int (&H)[3], long long site, long long pstride, typename P::cplx* S_out = nullptr,
-    const float4* bpre = nullptr, const typename PlaneLinkOf<P>::type* lk = nullptr,
     const int* Ngrid_p = nullptr) {
   // grid extent (cells per axis) for the soft-core correction index
   const int Ngrid[3] = {Ngrid_p ? Ngrid_p[0] : 1, Ngrid_p ? Ngrid_p[1] : 1, Ngrid_p ? Ngrid_p[2] : 1};
@@ -761,9 +756,8 @@ __device__ __forceinline__ typename P::cplx site_update(
       up = link_mul(h.L[ax], up);
       dn = link_mulc(h.L[ax], dn);
     } else if (link == LINK_TABLE) {
-      const long long i = (long long)plane * h.larr_ps + site;
-      up = link_mul(h.larr[(2 * ax) * h.larr_n + i], up);
-      dn = link_mulc(h.larr[(2 * ax + 1) * h.larr_n + i], dn);
+      up = link_mul(table_link<DIMS>(h, 2 * ax, plane, site), up);
+      dn = link_mulc(table_link<DIMS>(h, 2 * ax + 1, plane, site), dn);
     } else if (LINK == kAnyMode && (link == LINK_GENERAL || link == LINK_PLANE)) {
       long long HH[3] = {H[0], H[1], H[2]};
       up = link_mul(link_from(link_phase_site(f, DIMS, HH, ax, +1, h.t, plane, site), (P*)nullptr), up);
@@ -772,20 +766,12 @@ __device__ __forceinline__ typename P::cplx site_update(
     }
     d[ax] = csub(up, dn);
   }
-  if constexpr (LINK == LINK_PLANE_ZX) {
-    d[0] = plane_link_diff(*lk, nb[0], nb[1]);  // the factor of the value's z level, staged by the caller
-  }
   if constexpr (LINK == LINK_PLANE) {
     // the difference along the polarisation with the shared link factor of the
-    // value's neighbours: staged by the caller (lk), or from the step's table
+    // value's neighbours, from the step's table
     using PL = typename PlaneLinkOf<P>::type;
-    PL L;
-    if (lk) {
-      L = *lk;
-    } else {
-      const int hk = h.ltab_axis == 0 ? H[0] : (h.ltab_axis == 1 ? H[1] : H[2]);
-      L = static_cast<const PL*>(h.ltab)[hk];
-    }
+    const int hk = h.ltab_axis == 0 ? H[0] : (h.ltab_axis == 1 ? H[1] : H[2]);
+    const PL L = static_cast<const PL*>(h.ltab)[hk];
     if (h.lpol == 0) d[0] = plane_link_diff(L, nb[0], nb[1]);
     else if (h.lpol == 1) d[1] = plane_link_diff(L, nb[2], nb[3]);
     else if (DIMS == 3) d[2] = plane_link_diff(L, nb[4], nb[5]);
@@ -799,9 +785,9 @@ __device__ __forceinline__ typename P::cplx site_update(
     return hs >= h.step_X ? apply(h.c_out, F, S) : apply(h.c_in, F, S);
   }
   if (coef == COEF_TABLE) return apply_table(h, F, S, plane, site);
-  if (coef == COEF_SOFTCORE) return apply_softcore<DIMS>(h, F, S, H, bpre);
+  if (coef == COEF_SOFTCORE) return apply_softcore<DIMS>(h, F, S, H);
   if (coef == COEF_SOFTCORR) {
-    if constexpr (sizeof(typename P::real) == 4) return apply_softcorr_f32<DIMS>(h, F, S, H, bpre, plane, Ngrid);
+    if constexpr (sizeof(typename P::real) == 4) return apply_softcorr_f32<DIMS>(h, F, S, H, plane, Ngrid);
     else return F;  // not used: FP64 kernels take the general path
   }
   double V = potential_at(f, DIMS, H[0], H[1], H[2], site, pstride, plane, h.t);

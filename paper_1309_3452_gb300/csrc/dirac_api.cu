@@ -36,7 +36,8 @@ struct dirac_sim {
   size_t elem = 0;            // bytes per complex value
   void* state = nullptr;      // np * pstride values: the current state
   void* state_alt = nullptr;  // second buffer for the out-of-place fused kernels
-  int fused = 0;              // one kernel per time step (FP32 without the reference flag)
+  int fused = 0;              // one kernel per time step (FP32 without the reference flag); the state
+                              // (and the per-site tables) are then held as quads (quad.cuh)
   int tblock = 1;             // (2+1)D fused path: two time steps per pass when possible
   int chunk1 = 0, chunk2 = 0; // launch plan: levels per item (one-step / two-step kernel), 0 = rule
   double plan_us = 0;         // time per step the autotuner measured for the plan
@@ -293,7 +294,13 @@ static HalfFields<P> half_fields(const dirac_sim* s, bool upper, double t) {
   h.t = t;
   h.beta = beta;
   // tabulated potential
-  for (int k = 0; k < 8; ++k) h.b_tab[k] = s->b_tab && k < s->np ? s->b_tab + (long long)k * s->pstride : nullptr;
+  for (int k = 0; k < 8; ++k)
+    h.b_tab[k] = s->b_tab && !s->fused && k < s->np ? s->b_tab + (long long)k * s->pstride : nullptr;
+  if (s->fused) {
+    h.bq = s->b_tab;
+    h.lq = s->link_mode == LINK_TABLE ? reinterpret_cast<const float4*>(s->larr) : nullptr;
+    h.q_ps = s->pstride;
+  }
   split(rx, h.rx_hi, h.rx_lo);
   // analytic soft core: theta_0 on both sides of the Klein step, K = -dt Z/2
   // and the per-axis square tables (axis a at offset 2 (N_0 + ... + N_{a-1}))
@@ -311,7 +318,7 @@ static HalfFields<P> half_fields(const dirac_sim* s, bool upper, double t) {
     }
     h.sc_corr = s->sc_corr;
   }
-  if (s->link_mode == LINK_TABLE) {
+  if (s->link_mode == LINK_TABLE && !s->fused) {
     h.larr = reinterpret_cast<const typename P::Link*>(s->larr);
     h.larr_n = (long long)s->np * s->pstride;
     h.larr_ps = s->pstride;
@@ -350,12 +357,9 @@ template <class P>
 static FusedArgs<P> fused_args(dirac_sim* s, double t) {
   FusedArgs<P> a;
   std::memset(&a, 0, sizeof(a));
-  typename P::cplx* in[8];
-  plane_ptrs<P>(s, in);
-  auto* alt = static_cast<typename P::cplx*>(s->state_alt);
-  for (int k = 0; k < 8; ++k) {
-    a.in[k] = in[k];
-    a.out[k] = k < s->np ? alt + (long long)k * s->pstride : nullptr;
+  for (int c = 0; c < s->np / 2; ++c) {
+    a.in[c] = static_cast<const float4*>(s->state) + (long long)c * s->pstride;
+    a.out[c] = static_cast<float4*>(s->state_alt) + (long long)c * s->pstride;
   }
   for (int k = 0; k < 3; ++k) a.N[k] = s->N[k];
   a.pstride = s->pstride;
@@ -619,7 +623,7 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
       return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link factor table)"));
     if ((e = cudaMemsetAsync(s->larr, 0, tb, s->stream)) != cudaSuccess)
       return cleanup_fail(cuda_fail(s, e, "cudaMemsetAsync(link factor table)"));
-    launch_link_factor_table(s->larr, field_desc(s), dims, s->N, s->pstride, s->stream);
+    launch_link_factor_table(s->larr, field_desc(s), dims, s->N, s->pstride, s->fused, s->stream);
     if ((e = cudaGetLastError()) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "link factor table"));
     s->launches += 1;
   }
@@ -662,7 +666,7 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
   if (s->coef_mode == COEF_TABLE) {
     if ((e = cudaMalloc(&s->b_tab, (size_t)s->np * s->pstride * sizeof(float4))) != cudaSuccess)
       return cleanup_fail(cuda_fail(s, e, "cudaMalloc(coefficient table)"));
-    launch_coef_table(s->b_tab, field_desc(s), dims, s->N, s->pstride, s->stream);
+    launch_coef_table(s->b_tab, field_desc(s), dims, s->N, s->pstride, s->fused, s->stream);
     if ((e = cudaGetLastError()) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "coefficient table"));
     s->launches += 1;
   }
@@ -754,6 +758,63 @@ static const void* mapped_host(const void* p, size_t bytes) {
   return a0.devicePointer;
 }
 
+// the quads of component c of the current state (fused simulations)
+static float4* quads_of(const dirac_sim* s, int c) {
+  return static_cast<float4*>(s->state) + (long long)c * s->pstride;
+}
+
+// Canonical planes in memory the device can read (its own, or a mapped host
+// buffer) -> the state of an FP32 simulation
+static dirac_status convert_state_in(dirac_sim* s, const double2* src) {
+  if (s->fused) {
+    for (int c = 0; c < s->np / 2; ++c) {
+      launch_convert_in_quads(src + 2LL * c * s->ncell, src + (2LL * c + 1) * s->ncell, quads_of(s, c), -1, s->ncell,
+                              s->stream);
+      s->launches += 1;
+      CK(s, cudaGetLastError());
+    }
+    return DIRAC_OK;
+  }
+  for (int k = 0; k < s->np; ++k) {
+    launch_convert_in(src + (long long)k * s->ncell, static_cast<float2*>(s->state) + (long long)k * s->pstride,
+                      s->ncell, s->stream);
+    s->launches += 1;
+    CK(s, cudaGetLastError());
+  }
+  return DIRAC_OK;
+}
+// the state of an FP32 simulation -> canonical planes the device can write
+static dirac_status convert_state_out(dirac_sim* s, double2* dst) {
+  if (s->fused) {
+    for (int c = 0; c < s->np / 2; ++c) {
+      launch_convert_out_quads(quads_of(s, c), dst + 2LL * c * s->ncell, dst + (2LL * c + 1) * s->ncell, -1, s->ncell,
+                               s->stream);
+      s->launches += 1;
+      CK(s, cudaGetLastError());
+    }
+    return DIRAC_OK;
+  }
+  for (int k = 0; k < s->np; ++k) {
+    launch_convert_out(static_cast<const float2*>(s->state) + (long long)k * s->pstride,
+                       dst + (long long)k * s->ncell, s->ncell, s->stream);
+    s->launches += 1;
+    CK(s, cudaGetLastError());
+  }
+  return DIRAC_OK;
+}
+// one canonical plane in the staging buffer <-> plane k of an FP32 state
+static void staged_plane_in(dirac_sim* s, int k) {
+  if (s->fused) launch_convert_in_quads(s->staging, nullptr, quads_of(s, k >> 1), k & 1, s->ncell, s->stream);
+  else launch_convert_in(s->staging, static_cast<float2*>(s->state) + (long long)k * s->pstride, s->ncell, s->stream);
+  s->launches += 1;
+}
+static void staged_plane_out(dirac_sim* s, int k) {
+  if (s->fused) launch_convert_out_quads(quads_of(s, k >> 1), s->staging, nullptr, k & 1, s->ncell, s->stream);
+  else launch_convert_out(static_cast<const float2*>(s->state) + (long long)k * s->pstride, s->staging, s->ncell,
+                          s->stream);
+  s->launches += 1;
+}
+
 extern "C" dirac_status dirac_set_spinor(dirac_sim* s, const double* host) {
   if (!s || !host) return fail(s, DIRAC_ERR_INVALID, "NULL argument");
   s->e_valid_at = -1;
@@ -763,20 +824,19 @@ extern "C" dirac_status dirac_set_spinor(dirac_sim* s, const double* host) {
   const double2* mapped = s->prec == DIRAC_FP32
                               ? static_cast<const double2*>(mapped_host(host, bytes * (size_t)s->np))
                               : nullptr;
+  if (mapped) {
+    dirac_status st = convert_state_in(s, mapped);
+    if (st != DIRAC_OK) return st;
+    return take_reference(s);
+  }
   for (int k = 0; k < s->np; ++k) {
     const double* src = host + 2LL * k * s->ncell;
     if (s->prec == DIRAC_FP64) {
       double2* dst = static_cast<double2*>(s->state) + (long long)k * s->pstride;
       CK(s, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s->stream));
     } else {
-      float2* dst = static_cast<float2*>(s->state) + (long long)k * s->pstride;
-      if (mapped) {
-        launch_convert_in(mapped + (long long)k * s->ncell, dst, s->ncell, s->stream);
-      } else {
-        CK(s, cudaMemcpyAsync(s->staging, src, bytes, cudaMemcpyHostToDevice, s->stream));
-        launch_convert_in(s->staging, dst, s->ncell, s->stream);
-      }
-      s->launches += 1;
+      CK(s, cudaMemcpyAsync(s->staging, src, bytes, cudaMemcpyHostToDevice, s->stream));
+      staged_plane_in(s, k);
       CK(s, cudaGetLastError());
     }
   }
@@ -789,21 +849,21 @@ extern "C" dirac_status dirac_get_spinor(dirac_sim* s, double* host) {
   double2* mapped = s->prec == DIRAC_FP32
                         ? static_cast<double2*>(const_cast<void*>(mapped_host(host, bytes * (size_t)s->np)))
                         : nullptr;
+  if (mapped) {
+    dirac_status st = convert_state_out(s, mapped);
+    if (st != DIRAC_OK) return st;
+    CK(s, cudaStreamSynchronize(s->stream));
+    return DIRAC_OK;
+  }
   for (int k = 0; k < s->np; ++k) {
     double* dst = host + 2LL * k * s->ncell;
     if (s->prec == DIRAC_FP64) {
       const double2* src = static_cast<double2*>(s->state) + (long long)k * s->pstride;
       CK(s, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s->stream));
     } else {
-      const float2* src = static_cast<float2*>(s->state) + (long long)k * s->pstride;
-      if (mapped) {
-        launch_convert_out(src, mapped + (long long)k * s->ncell, s->ncell, s->stream);
-      } else {
-        launch_convert_out(src, s->staging, s->ncell, s->stream);
-      }
-      s->launches += 1;
+      staged_plane_out(s, k);
       CK(s, cudaGetLastError());
-      if (!mapped) CK(s, cudaMemcpyAsync(dst, s->staging, bytes, cudaMemcpyDeviceToHost, s->stream));
+      CK(s, cudaMemcpyAsync(dst, s->staging, bytes, cudaMemcpyDeviceToHost, s->stream));
     }
   }
   CK(s, cudaStreamSynchronize(s->stream));
@@ -816,38 +876,24 @@ extern "C" dirac_status dirac_set_spinor_device(dirac_sim* s, const void* dev) {
   if (!s || !dev) return fail(s, DIRAC_ERR_INVALID, "NULL argument");
   s->e_valid_at = -1;
   const double2* src = static_cast<const double2*>(dev);
-  for (int k = 0; k < s->np; ++k) {
-    const double2* plane = src + (long long)k * s->ncell;
-    if (s->prec == DIRAC_FP64) {
-      double2* dst = static_cast<double2*>(s->state) + (long long)k * s->pstride;
-      CK(s, cudaMemcpyAsync(dst, plane, (size_t)s->ncell * sizeof(double2), cudaMemcpyDeviceToDevice,
-                            s->stream));
-    } else {
-      launch_convert_in(plane, static_cast<float2*>(s->state) + (long long)k * s->pstride, s->ncell,
-                        s->stream);
-      s->launches += 1;
-      CK(s, cudaGetLastError());
-    }
+  if (s->prec == DIRAC_FP32) {
+    dirac_status st = convert_state_in(s, src);
+    if (st != DIRAC_OK) return st;
+    return take_reference(s);
   }
+  for (int k = 0; k < s->np; ++k)
+    CK(s, cudaMemcpyAsync(static_cast<double2*>(s->state) + (long long)k * s->pstride, src + (long long)k * s->ncell,
+                          (size_t)s->ncell * sizeof(double2), cudaMemcpyDeviceToDevice, s->stream));
   return take_reference(s);
 }
 
 extern "C" dirac_status dirac_get_spinor_device(dirac_sim* s, void* dev) {
   if (!s || !dev) return fail(s, DIRAC_ERR_INVALID, "NULL argument");
   double2* dst = static_cast<double2*>(dev);
-  for (int k = 0; k < s->np; ++k) {
-    double2* plane = dst + (long long)k * s->ncell;
-    if (s->prec == DIRAC_FP64) {
-      const double2* src = static_cast<double2*>(s->state) + (long long)k * s->pstride;
-      CK(s, cudaMemcpyAsync(plane, src, (size_t)s->ncell * sizeof(double2), cudaMemcpyDeviceToDevice,
-                            s->stream));
-    } else {
-      launch_convert_out(static_cast<float2*>(s->state) + (long long)k * s->pstride, plane, s->ncell,
-                         s->stream);
-      s->launches += 1;
-      CK(s, cudaGetLastError());
-    }
-  }
+  if (s->prec == DIRAC_FP32) return convert_state_out(s, dst);
+  for (int k = 0; k < s->np; ++k)
+    CK(s, cudaMemcpyAsync(dst + (long long)k * s->ncell, static_cast<double2*>(s->state) + (long long)k * s->pstride,
+                          (size_t)s->ncell * sizeof(double2), cudaMemcpyDeviceToDevice, s->stream));
   return DIRAC_OK;
 }
 
@@ -1139,9 +1185,9 @@ static dirac_status batch_group(dirac_sim* const* g, int n, long nsteps) {
         FusedArgs<F32> a = fused_args<F32>(s, sim_time(s));
         a.chunk = chunks[2 * i + mode];
         if (p == 1) {
-          for (int k = 0; k < 8; ++k) {  // the other buffer is the input after an odd launch
-            typename F32::cplx* tmp = a.out[k];
-            a.out[k] = const_cast<typename F32::cplx*>(a.in[k]);
+          for (int k = 0; k < 4; ++k) {  // the other buffer is the input after an odd launch
+            float4* tmp = a.out[k];
+            a.out[k] = const_cast<float4*>(a.in[k]);
             a.in[k] = tmp;
           }
         }
@@ -1275,7 +1321,10 @@ static dirac_status observe_launch(dirac_sim* s, int dens_axis, int dens_X, doub
   std::memset(&a, 0, sizeof(a));
   typename P::cplx* pl[8];
   plane_ptrs<P>(s, pl);
-  for (int k = 0; k < 8; ++k) a.pl[k] = pl[k];
+  if (s->fused)
+    for (int c = 0; c < s->np / 2; ++c) a.quads[c] = quads_of(s, c);
+  else
+    for (int k = 0; k < 8; ++k) a.pl[k] = pl[k];
   for (int k = 0; k < 3; ++k) a.N[k] = s->N[k];
   a.pstride = s->pstride;
   a.link_mode = s->link_mode;
@@ -1666,14 +1715,14 @@ extern "C" dirac_status dirac_slabs_info(const dirac_slabs* g, int k, int* z0, i
   return DIRAC_OK;
 }
 
-// copy one stored level of every plane from slab a into slab b (device to
+// copy one stored level of every component from slab a into slab b (device to
 // device on the group's stream)
 static dirac_status copy_level(dirac_slabs* g, dirac_sim* a, int la, dirac_sim* b, int lb) {
   const size_t lvl = g->march == 2 ? (size_t)a->N[0] * a->N[1] : (size_t)a->N[0];  // values per level
-  for (int p = 0; p < a->np; ++p) {
-    const float2* src = static_cast<const float2*>(a->state) + (long long)p * a->pstride + (long long)la * lvl;
-    float2* dst = static_cast<float2*>(b->state) + (long long)p * b->pstride + (long long)lb * lvl;
-    cudaError_t e = cudaMemcpyAsync(dst, src, lvl * sizeof(float2), cudaMemcpyDeviceToDevice, g->stream);
+  for (int c = 0; c < a->np / 2; ++c) {
+    const float4* src = quads_of(a, c) + (long long)la * lvl;
+    float4* dst = quads_of(b, c) + (long long)lb * lvl;
+    cudaError_t e = cudaMemcpyAsync(dst, src, lvl * sizeof(float4), cudaMemcpyDeviceToDevice, g->stream);
     if (e != cudaSuccess) return slabs_fail(g, DIRAC_ERR_CUDA, std::string("halo copy: ") + cudaGetErrorString(e));
   }
   return DIRAC_OK;
@@ -1711,8 +1760,7 @@ extern "C" dirac_status dirac_slabs_set_spinor(dirac_slabs* g, const double* hos
                                         s->stream);
         if (e != cudaSuccess) return slabs_fail(g, DIRAC_ERR_CUDA, std::string("set: ") + cudaGetErrorString(e));
       }
-      launch_convert_in(s->staging, static_cast<float2*>(s->state) + (long long)p * s->pstride, s->ncell, s->stream);
-      s->launches += 1;
+      staged_plane_in(s, p);
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return slabs_fail(g, DIRAC_ERR_CUDA, std::string("set: ") + cudaGetErrorString(e));
     }
@@ -1729,9 +1777,7 @@ extern "C" dirac_status dirac_slabs_get_spinor(dirac_slabs* g, double* host) {
   for (int k = 0; k < g->n; ++k) {
     dirac_sim* s = g->sim[k];
     for (int p = 0; p < s->np; ++p) {
-      launch_convert_out(static_cast<const float2*>(s->state) + (long long)p * s->pstride, s->staging, s->ncell,
-                         s->stream);
-      s->launches += 1;
+      staged_plane_out(s, p);
       cudaError_t e = cudaGetLastError();
       // own levels 1 .. nz only
       if (e == cudaSuccess)

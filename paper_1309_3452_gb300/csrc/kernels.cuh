@@ -1,6 +1,8 @@
 // Kernel argument blocks and launcher declarations of libdirac.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace dirac {
@@ -24,8 +26,8 @@ void launch_half_step(const HalfStepArgs<P>& a, bool upper, cudaStream_t s);
 // One full time step (both half-steps) in one kernel, out of place.
 template <class P>
 struct FusedArgs {
-  const typename P::cplx* in[8];
-  typename P::cplx* out[8];
+  const float4* in[4];      // components (quad.cuh): A, B, C, D or u, v
+  float4* out[4];
   int N[3];
   int chunk;                // levels (z in (3+1)D, y in (2+1)D) per work item
   int workers;              // persistent workers: blocks ((3+1)D) or warps ((2+1)D)
@@ -94,6 +96,7 @@ void launch_fused2d_tb2_batch(const BatchArgs<F32>& b, long long total_items, in
 template <class P>
 struct ObsArgs {
   const typename P::cplx* pl[8];
+  const float4* quads[4];   // F32 states held as quads (quad.cuh), else null
   int N[3];
   long long pstride;
   int link_mode;
@@ -124,8 +127,8 @@ void launch_link_table(void* tab, int n, const FieldDesc& f, int dims, int axis,
 
 // coefficient table of a time-independent potential (COEF_TABLE): every
 // plane of the state layout (pstride), b = 1/(1 + i dt (beta m + V)/2) as
-// {re hi, im hi, re lo, im lo}
-void launch_coef_table(float4* tab, const FieldDesc& f, int dims, const int N[3], long long pstride,
+// {re hi, im hi, re lo, im lo}, or (quads) as the quad records of quad.cuh
+void launch_coef_table(float4* tab, const FieldDesc& f, int dims, const int N[3], long long pstride, int quads,
                        cudaStream_t s);
 
 // COEF_SOFTCORR correction records of a soft-core potential (one 32-bit word
@@ -143,9 +146,10 @@ void launch_link_integral_table(double* out, const double* raw, int dims, const 
 
 // LINK_TABLE: exp(-i phi) of every value's up link (slot 2a) and down link
 // (slot 2a+1) of a time-independent vector potential, FP32 hi + lo pairs:
-// out[slot * P * pstride + plane * pstride + cell]
+// out[slot * P * pstride + plane * pstride + cell], or (quads) as the quad
+// records of quad.cuh, slot by slot
 void launch_link_factor_table(F32::Link* out, const FieldDesc& f, int dims, const int N[3], long long pstride,
-                              cudaStream_t s);
+                              int quads, cudaStream_t s);
 
 // measured FP64 FMA rate of the current device (TFLOP/s), < 0 on a CUDA failure
 double measure_fp64_fma_tflops();
@@ -153,5 +157,11 @@ double measure_fp64_fma_tflops();
 // canonical complex128 plane <-> device plane of the simulation precision
 void launch_convert_in(const double2* src, float2* dst, long long n, cudaStream_t s);
 void launch_convert_out(const float2* src, double2* dst, long long n, cudaStream_t s);
+// the same for states held as quads: two planes <-> one component (lane < 0),
+// or one plane <-> that sublattice of it (lane 0 or 1: src0 / dst0)
+void launch_convert_in_quads(const double2* src0, const double2* src1, float4* dst, int lane, long long n,
+                             cudaStream_t s);
+void launch_convert_out_quads(const float4* src, double2* dst0, double2* dst1, int lane, long long n,
+                              cudaStream_t s);
 
 }  // namespace dirac

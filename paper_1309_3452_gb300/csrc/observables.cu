@@ -6,6 +6,7 @@
 // per warp (shuffles), per block (shared memory) and finally over blocks in a
 // fixed order, so the result is deterministic for a given grid.
 #include "kernels.cuh"
+#include "quad.cuh"
 
 namespace dirac {
 
@@ -49,6 +50,17 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NS], double* out)
 // states: every term is a product of two stored floats, rounded once; the
 // FP64 accumulation over cells keeps the sum accurate), except with
 // plane-wave link factors, which are evaluated in FP64.
+template <class P>
+__device__ __forceinline__ typename P::cplx obs_value(const ObsArgs<P>& a, int plane, long long cell) {
+  return a.pl[plane][cell];
+}
+template <>
+__device__ __forceinline__ float2 obs_value(const ObsArgs<F32>& a, int plane, long long cell) {
+  if (!a.quads[0]) return a.pl[plane][cell];
+  const float* r = reinterpret_cast<const float*>(a.quads[plane >> 1] + cell) + (plane & 1);
+  return make_float2(r[0], r[2]);
+}
+
 template <class P, int DIMS>
 __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
   using C = typename P::cplx;
@@ -80,7 +92,7 @@ __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
       R cn = 0, cd = 0, cb[3] = {0, 0, 0};
 #pragma unroll
       for (int plane = 0; plane < nplanes<DIMS>(); ++plane) {
-        const C G = a.pl[plane][cell];
+        const C G = obs_value(a, plane, cell);
         const R n2 = G.x * G.x + G.y * G.y;
         cn += n2;
         long long H[3];
@@ -93,13 +105,13 @@ __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
         const int p = sign_class<DIMS>(plane);
 #pragma unroll
         for (int ax = 0; ax < DIMS; ++ax) {
-          const C* nb = a.pl[partner<DIMS>(plane, ax)];
+          const int pn = partner<DIMS>(plane, ax);
           int jp = j[ax] + nb_shift<DIMS>(plane, ax, +1);
           int jm = j[ax] + nb_shift<DIMS>(plane, ax, -1);
           jp = jp >= Nn[ax] ? jp - Nn[ax] : jp;
           jm = jm < 0 ? jm + Nn[ax] : jm;
-          C up = nb[cell + (long long)(jp - j[ax]) * stride[ax]];
-          C dn = nb[cell + (long long)(jm - j[ax]) * stride[ax]];
+          C up = obs_value(a, pn, cell + (long long)(jp - j[ax]) * stride[ax]);
+          C dn = obs_value(a, pn, cell + (long long)(jm - j[ax]) * stride[ax]);
           R re, im;
           if (a.link_mode == LINK_PLANE) {
             // a plane wave with its wave vector across the polarisation (and no
@@ -177,6 +189,17 @@ __device__ __forceinline__ void plane_link_from(double phi, PlaneLink32* out) {
   out->cl = make_float2(cl, cl);
   out->sh = make_float2(sh, -sh);
   out->sl = make_float2(sl, -sl);
+  out->sp = make_float2(sh, sh);
+  out->lp = make_float2(sl, sl);
+}
+
+// one value's {re hi, im hi, re lo, im lo} into a quad record
+__device__ __forceinline__ void store_quad_lane(float4* rec, int lane, float4 v) {
+  float* r = reinterpret_cast<float*>(rec) + lane;
+  r[0] = v.x;
+  r[2] = v.y;
+  r[4] = v.z;
+  r[6] = v.w;
 }
 
 template <class P>
@@ -197,7 +220,7 @@ __global__ void link_table_kernel(typename PlaneLinkOf<P>::type* tab, int n, con
 // potentials only); stored as {re hi, im hi, re lo, im lo}
 template <int DIMS>
 __global__ void coef_table_kernel(float4* __restrict__ tab, const FieldDesc f, int N0, int N1, int N2,
-                                  long long pstride) {
+                                  long long pstride, int quads) {
   const int plane = blockIdx.y;
   const long long ncell = (long long)N0 * N1 * N2;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
@@ -213,8 +236,9 @@ __global__ void coef_table_kernel(float4* __restrict__ tab, const FieldDesc f, i
     const double k = 1.0 / ((1.0 - tb) * (1.0 - tb) + ta * ta);
     const double re = (1.0 - tb) * k, im = -ta * k;
     const float rh = __double2float_rn(re), ih = __double2float_rn(im);
-    tab[plane * pstride + c] =
-        make_float4(rh, ih, __double2float_rn(re - (double)rh), __double2float_rn(im - (double)ih));
+    const float4 b = make_float4(rh, ih, __double2float_rn(re - (double)rh), __double2float_rn(im - (double)ih));
+    if (quads) store_quad_lane(tab + 2 * ((plane >> 1) * pstride + c), plane & 1, b);
+    else tab[plane * pstride + c] = b;
   }
 }
 
@@ -296,7 +320,7 @@ __global__ void link_integral_table_kernel(double* __restrict__ out, const doubl
 // (dir 0: the value's up link; dir 1: the link from its lower neighbour)
 template <int DIMS>
 __global__ void link_factor_table_kernel(F32::Link* __restrict__ out, const FieldDesc f, int N0, int N1, int N2,
-                                         long long pstride) {
+                                         long long pstride, int quads) {
   const int plane = blockIdx.y, slot = blockIdx.z, axis = slot >> 1, dir = (slot & 1) ? -1 : 1;
   const long long ncell = (long long)N0 * N1 * N2;
   const long long n = (long long)nplanes<DIMS>() * pstride;
@@ -306,7 +330,11 @@ __global__ void link_factor_table_kernel(F32::Link* __restrict__ out, const Fiel
     const long long H[3] = {2 * x + plane_off<DIMS>(plane, 0), 2 * y + plane_off<DIMS>(plane, 1),
                             DIMS == 3 ? 2 * z + plane_off<DIMS>(plane, 2) : 0};
     const double phi = link_phase_site(f, DIMS, H, axis, dir, 0.0, plane, c);
-    out[slot * n + plane * pstride + c] = link_from(phi, (F32*)nullptr);
+    const F32::Link L = link_from(phi, (F32*)nullptr);
+    if (quads)  // the quads of slot, component: 2 * ((slot * components + component) * pstride + cell)
+      store_quad_lane(reinterpret_cast<float4*>(out) + slot * n + 2 * ((plane >> 1) * pstride + c), plane & 1,
+                      make_float4(L.hi.x, L.hi.y, L.lo.x, L.lo.y));
+    else out[slot * n + plane * pstride + c] = L;
   }
 }
 
@@ -332,6 +360,38 @@ __global__ void convert_out_kernel(const float2* __restrict__ src, double2* __re
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     dst[i] = make_double2(src[i].x, src[i].y);
+}
+
+// two canonical planes <-> one component's quads; lane < 0: both planes, else
+// the one plane of that sublattice (src0 / dst0)
+__global__ void convert_in_quads_kernel(const double2* __restrict__ src0, const double2* __restrict__ src1,
+                                        float4* __restrict__ dst, int lane, long long n) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const double2 v = src0[i];
+    const float re = __double2float_rn(v.x), im = __double2float_rn(v.y);
+    if (lane < 0) {
+      const double2 w = src1[i];
+      dst[i] = make_float4(re, __double2float_rn(w.x), im, __double2float_rn(w.y));
+    } else {
+      float* r = reinterpret_cast<float*>(dst + i) + lane;
+      r[0] = re;
+      r[2] = im;
+    }
+  }
+}
+__global__ void convert_out_quads_kernel(const float4* __restrict__ src, double2* __restrict__ dst0,
+                                         double2* __restrict__ dst1, int lane, long long n) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const float4 q = src[i];
+    if (lane < 0) {
+      dst0[i] = make_double2(q.x, q.z);
+      dst1[i] = make_double2(q.y, q.w);
+    } else {
+      dst0[i] = lane ? make_double2(q.y, q.w) : make_double2(q.x, q.z);
+    }
+  }
 }
 
 // FP64 FMA throughput: eight independent dependency chains of fused
@@ -414,16 +474,16 @@ void launch_link_table(void* tab, int n, const FieldDesc& f, int dims, int axis,
 template void launch_link_table<F64>(void*, int, const FieldDesc&, int, int, int, double, double, cudaStream_t);
 template void launch_link_table<F32>(void*, int, const FieldDesc&, int, int, int, double, double, cudaStream_t);
 
-void launch_coef_table(float4* tab, const FieldDesc& f, int dims, const int N[3], long long pstride,
+void launch_coef_table(float4* tab, const FieldDesc& f, int dims, const int N[3], long long pstride, int quads,
                        cudaStream_t s) {
   const long long ncell = (long long)N[0] * N[1] * (dims == 3 ? N[2] : 1);
   long long bx = (ncell + 255) / 256;
   if (bx > 152 * 16) bx = 152 * 16;
   const dim3 grid((unsigned)bx, dims == 3 ? 8 : 4);
   if (dims == 3)
-    coef_table_kernel<3><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], N[2], pstride);
+    coef_table_kernel<3><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], N[2], pstride, quads);
   else
-    coef_table_kernel<2><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], 1, pstride);
+    coef_table_kernel<2><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], 1, pstride, quads);
 }
 
 void launch_softcore_corr(unsigned* out, const HalfFields<F32>& hu, const HalfFields<F32>& hl, const FieldDesc& f,
@@ -450,15 +510,15 @@ void launch_link_integral_table(double* out, const double* raw, int dims, const 
 }
 
 void launch_link_factor_table(F32::Link* out, const FieldDesc& f, int dims, const int N[3], long long pstride,
-                              cudaStream_t s) {
+                              int quads, cudaStream_t s) {
   const long long ncell = (long long)N[0] * N[1] * (dims == 3 ? N[2] : 1);
   long long bx = (ncell + 255) / 256;
   if (bx > 152 * 16) bx = 152 * 16;
   const dim3 grid((unsigned)bx, dims == 3 ? 8 : 4, 2 * dims);
   if (dims == 3)
-    link_factor_table_kernel<3><<<grid, 256, 0, s>>>(out, f, N[0], N[1], N[2], pstride);
+    link_factor_table_kernel<3><<<grid, 256, 0, s>>>(out, f, N[0], N[1], N[2], pstride, quads);
   else
-    link_factor_table_kernel<2><<<grid, 256, 0, s>>>(out, f, N[0], N[1], 1, pstride);
+    link_factor_table_kernel<2><<<grid, 256, 0, s>>>(out, f, N[0], N[1], 1, pstride, quads);
 }
 
 void launch_finish_sums2(const double* partials, int nblocks, double* out, cudaStream_t s) {
@@ -478,6 +538,14 @@ void launch_convert_in(const double2* src, float2* dst, long long n, cudaStream_
 }
 void launch_convert_out(const float2* src, double2* dst, long long n, cudaStream_t s) {
   convert_out_kernel<<<grid_for(n), 256, 0, s>>>(src, dst, n);
+}
+void launch_convert_in_quads(const double2* src0, const double2* src1, float4* dst, int lane, long long n,
+                             cudaStream_t s) {
+  convert_in_quads_kernel<<<grid_for(n), 256, 0, s>>>(src0, src1, dst, lane, n);
+}
+void launch_convert_out_quads(const float4* src, double2* dst0, double2* dst1, int lane, long long n,
+                              cudaStream_t s) {
+  convert_out_quads_kernel<<<grid_for(n), 256, 0, s>>>(src, dst0, dst1, lane, n);
 }
 
 }  // namespace dirac

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(128) half_step_kernel(const HalfStepArgs<P> a)
       }
     }
     self[cell] = site_update<P, DIMS, COEF, LINK>(a.h, a.f, a.iso != 0, a.ry, a.rz, plane, self[cell],
-                                               nb, H, cell, a.pstride, nullptr, nullptr, nullptr, a.N);
+                                               nb, H, cell, a.pstride, nullptr, a.N);
   }
 }
 
