@@ -60,6 +60,7 @@ struct dirac_sim {
   int coef_mode = COEF_UNIFORM, link_mode = LINK_NONE;
   int step_X = 0;
   void* ltab = nullptr;       // LINK_PLANE: link-factor table of the current step
+  void* wave = nullptr;       // LINK_PLANE: link-factor table of the reductions
   int ltab_axis = 0, ltab_n = 0;
   long long launches = 0;     // kernels launched so far
   // CUDA graphs of kGraphSteps time steps, one per current-buffer parity
@@ -674,6 +675,8 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
     size_t tb = (size_t)2 * s->ltab_n * (precision == DIRAC_FP32 ? sizeof(PlaneLinkOf<F32>::type)
                                                                  : sizeof(PlaneLinkOf<F64>::type));
     if ((e = cudaMalloc(&s->ltab, tb)) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link table)"));
+    if ((e = cudaMalloc(&s->wave, tb)) != cudaSuccess)
+      return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link table)"));
   }
   if (s->fused) {
     if ((e = cudaMalloc(&s->e_partials, (size_t)kFusedEMaxBlocks * 2 * sizeof(double))) != cudaSuccess ||
@@ -721,6 +724,7 @@ extern "C" void dirac_destroy(dirac_sim* s) {
   cudaFree(s->Alink);
   cudaFree(s->larr);
   cudaFree(s->ltab);
+  cudaFree(s->wave);
   cudaFree(s->e_partials);
   cudaFree(s->e_sums);
   cudaFree(s->partials);
@@ -1331,6 +1335,15 @@ static dirac_status observe_launch(dirac_sim* s, int dens_axis, int dens_X, doub
   for (int k = 0; k < 3; ++k) a.L[k] = make_link<P>(s->f.q * s->f.A_const[k] * s->dx[k] / 2.0);
   a.f = field_desc(s);
   a.t_links = sim_time(s) - s->dt / 2.0;
+  if (s->link_mode == LINK_PLANE) {
+    launch_link_table<P>(s->wave, s->ltab_n, a.f, s->dims, s->ltab_axis, s->f.Apw_pol, a.t_links, a.t_links,
+                         s->stream);
+    s->launches += 1;
+    CK(s, cudaGetLastError());
+    a.wave = s->wave;
+    a.wave_axis = s->ltab_axis;
+  }
+  if (s->link_mode == LINK_TABLE && s->fused) a.lq = reinterpret_cast<const float4*>(s->larr);
   a.dens_axis = dens_axis;
   a.dens_X = dens_X;
   a.partials = s->partials;
@@ -1338,10 +1351,10 @@ static dirac_status observe_launch(dirac_sim* s, int dens_axis, int dens_X, doub
   a.nzu = s->nzu;
   a.zorg = s->zorg;
   a.Nzg = s->Nzg;
-  if (s->dims == 3) launch_observables<P, 3>(a, s->red_blocks, s->stream);
-  else launch_observables<P, 2>(a, s->red_blocks, s->stream);
+  const int blocks = s->dims == 3 ? launch_observables<P, 3>(a, s->red_blocks, s->stream)
+                                  : launch_observables<P, 2>(a, s->red_blocks, s->stream);
   CK(s, cudaGetLastError());
-  launch_finish_sums(s->partials, s->red_blocks, out_dev, s->stream);
+  launch_finish_sums(s->partials, blocks, out_dev, s->stream);
   s->launches += 2;
   CK(s, cudaGetLastError());
   return DIRAC_OK;

@@ -103,16 +103,23 @@ struct ObsArgs {
   typename P::Link L[3];
   FieldDesc f;
   double t_links;           // time of the upper sheet (t - dt/2)
+  // LINK_PLANE: the link factors at t_links by half-lattice coordinate along the
+  // wave vector, PlaneLinkOf<P> (null: phases evaluated per link); LINK_TABLE
+  // of quads
+  const void* wave;
+  int wave_axis;
+  const float4* lq;
   int dens_axis, dens_X;    // partial density: half-lattice index >= dens_X along axis
   double* partials;         // [gridDim.x][5]
   int zlo, nzu, zorg, Nzg;  // levels summed along the marching axis and their global position, as in FusedArgs
 };
 constexpr int kObsSums = 5;
 
-// number of blocks (= partial sums) the observables kernel uses for a grid
+// the most blocks (= partial sums) the observables kernel uses for a grid;
+// the launcher returns how many ran
 int observables_blocks(const int N[3], int dims);
 template <class P, int DIMS>
-void launch_observables(const ObsArgs<P>& a, int blocks, cudaStream_t s);
+int launch_observables(const ObsArgs<P>& a, int blocks, cudaStream_t s);
 // fixed-order sum of partials[nblocks][5] into out[5]
 void launch_finish_sums(const double* partials, int nblocks, double* out, cudaStream_t s);
 // fixed-order sum of partials[nblocks][2] into out[2]

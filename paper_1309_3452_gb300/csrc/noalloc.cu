@@ -68,7 +68,7 @@ template <> F32::Link noalloc_link<F32>(double phi) {
 }
 
 template <class P>
-void launch(int dims, const int N[3], const double dx[3], double dt, double t,
+int launch(int dims, const int N[3], const double dx[3], double dt, double t,
             const dirac_fields& f, const void* const* planes, double* scratch, int blocks,
             cudaStream_t s) {
   ObsArgs<P> a;
@@ -88,8 +88,7 @@ void launch(int dims, const int N[3], const double dx[3], double dt, double t,
   a.zlo = 0;
   a.nzu = a.Nzg = dims == 3 ? a.N[2] : a.N[1];  // every level of the marching axis
   a.zorg = 0;
-  if (dims == 3) launch_observables<P, 3>(a, blocks, s);
-  else launch_observables<P, 2>(a, blocks, s);
+  return dims == 3 ? launch_observables<P, 3>(a, blocks, s) : launch_observables<P, 2>(a, blocks, s);
 }
 
 }  // namespace
@@ -117,8 +116,10 @@ extern "C" dirac_status dirac_norm_noalloc(int dims, const int N[3], const doubl
     if (!std::isfinite(v)) return DIRAC_ERR_INVALID;
   if (f.Apw_amp != 0.0 && (f.Apw_pol < 0 || f.Apw_pol >= dims)) return DIRAC_ERR_INVALID;
   // the reduction grid of this size must fit the fixed scratch array
-  const int blocks = observables_blocks(N, dims);
-  if (blocks > kNoAllocMaxBlocks) return DIRAC_ERR_UNSUPPORTED;
+  // (the documented limit; the reduction itself uses fewer blocks)
+  if ((long long)((N[0] + 31) / 32) * ((N[1] + 7) / 8) > kNoAllocMaxBlocks) return DIRAC_ERR_UNSUPPORTED;
+  const int n3[3] = {N[0], N[1], dims == 3 ? N[2] : 1};
+  const int blocks = observables_blocks(n3, dims);
 
   // The host-side name of the array is not a device address: ask the runtime
   // for the address of the current device's copy.  This allocates nothing
@@ -133,12 +134,10 @@ extern "C" dirac_status dirac_norm_noalloc(int dims, const int N[3], const doubl
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   // every reduction block overwrites its own partial slot and the final sums
   // are overwritten too, so nothing in the scratch needs clearing
-  if (precision == DIRAC_FP64)
-    launch<F64>(dims, N, dx, dt, t, f, planes, scratch, blocks, s);
-  else
-    launch<F32>(dims, N, dx, dt, t, f, planes, scratch, blocks, s);
+  const int used = precision == DIRAC_FP64 ? launch<F64>(dims, N, dx, dt, t, f, planes, scratch, blocks, s)
+                                           : launch<F32>(dims, N, dx, dt, t, f, planes, scratch, blocks, s);
   double* sums = scratch + (long long)kNoAllocMaxBlocks * kObsSums;
-  launch_finish_sums(scratch, blocks, sums, s);
+  launch_finish_sums(scratch, used, sums, s);
   combine_kernel<<<1, 32, 0, s>>>(sums, dt / dx[0], dt / dx[1], dims == 3 ? dt / dx[2] : 0.0, dims,
                                   out_dev);
   return cudaGetLastError() == cudaSuccess ? DIRAC_OK : DIRAC_ERR_CUDA;

@@ -1,12 +1,9 @@
 // Reductions of the stored state: the naive norm, the cross terms of the
 // conserved functional (Lemma of Sect. 2, Eq. EPM, in its "lower" form; see
-// dirac.h) and the partial density used for the Klein-step transmission.
-// One thread per cell (z strided over the grid's z blocks): the cell's terms
-// are summed in the state's precision, then accumulated in FP64 per thread,
-// per warp (shuffles), per block (shared memory) and finally over blocks in a
-// fixed order, so the result is deterministic for a given grid.
+// dirac.h) and the partial density used for the Klein-step transmission; and
+// the tables and layout conversions that a simulation is set up with.
 #include "kernels.cuh"
-#include "quad.cuh"
+#include "fused_common.cuh"
 
 namespace dirac {
 
@@ -46,133 +43,234 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NS], double* out)
   }
 }
 
-// Per-cell terms are formed in the working precision of the state (FP32
-// states: every term is a product of two stored floats, rounded once; the
-// FP64 accumulation over cells keeps the sum accurate), except with
-// plane-wave link factors, which are evaluated in FP64.
+// Running sums of a thread: FP64 for FP64 states.  For FP32 states the FP64
+// pipe (1.6 lanes per clock and SM) would be the limit, so a cell's terms are
+// added to an unevaluated sum hi + lo of two floats (TwoSum: the rounding error
+// of every addition is kept, relative error of the sum below 2^-44), which
+// goes to FP64 every kFlush cells: over the ~10^3 cells of a thread no less
+// exact than FP64 additions one by one.
+constexpr int kFlush = 16;
+struct Sum32 {
+  float h, l;
+  __device__ __forceinline__ void add(float v) {
+    const float s = __fadd_rn(h, v), b = __fsub_rn(s, h);
+    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(v, b)));
+    h = s;
+  }
+  // f v with f = fh + fl: the product's error by FMA
+  __device__ __forceinline__ void add_product(float fh, float fl, float v) {
+    const float p = __fmul_rn(fh, v);
+    l = __fmaf_rn(fl, v, __fadd_rn(l, __fmaf_rn(fh, v, -p)));
+    add(p);
+  }
+  __device__ __forceinline__ void flush(double& acc) {
+    acc += (double)h + (double)l;
+    h = l = 0.0f;
+  }
+};
+struct Sum64 {
+  double h;
+  __device__ __forceinline__ void add(double v) { h += v; }
+  __device__ __forceinline__ void flush(double& acc) {
+    acc += h;
+    h = 0.0;
+  }
+};
+template <class P> struct SumOf { using type = Sum64; };
+template <> struct SumOf<F32> { using type = Sum32; };
+
+// Both values of a component in one cell (two planes, or one quad).
 template <class P>
-__device__ __forceinline__ typename P::cplx obs_value(const ObsArgs<P>& a, int plane, long long cell) {
-  return a.pl[plane][cell];
-}
-template <>
-__device__ __forceinline__ float2 obs_value(const ObsArgs<F32>& a, int plane, long long cell) {
-  if (!a.quads[0]) return a.pl[plane][cell];
-  const float* r = reinterpret_cast<const float*>(a.quads[plane >> 1] + cell) + (plane & 1);
-  return make_float2(r[0], r[2]);
+struct Pair {
+  typename P::cplx v[2];
+};
+template <class P, bool kQuads>
+__device__ __forceinline__ Pair<P> load_pair(const ObsArgs<P>& a, int comp, long long cell) {
+  if constexpr (kQuads) {
+    const float4 q = __ldg(a.quads[comp] + cell);
+    return Pair<P>{{make_float2(q.x, q.z), make_float2(q.y, q.w)}};
+  } else {
+    return Pair<P>{{a.pl[2 * comp][cell], a.pl[2 * comp + 1][cell]}};
+  }
 }
 
-template <class P, int DIMS>
+// A warp takes 32 cells along x of one row at a time, rows dealt to a grid
+// that fills the GPU once.  Per cell the terms are formed in the state's
+// precision (FP32 states: products of two stored floats) and accumulated per
+// thread (SumOf), then in FP64 per warp (shuffles), per block and over the
+// blocks, in a fixed order, so the result is deterministic for a given grid.
+// Plane-wave link factors c - i s come from a table: the cross term of a value
+// is c P + s Q with P = Re conj(G) (up - dn) and Q = Re -i conj(G) (up + dn) in
+// the state's precision.  kLink: LINK_TABLE is the quads' table of factors; any
+// other vector potential (LINK_GENERAL) evaluates its phases in FP64.
+// Bound: loads (14 16-byte records per cell, about 5 from L2 or HBM).
+// us at 128^3 free / 4096^2 / 512^3 laser: with a block per 32 x 8 cells and z
+// range, a sincos per link, FP64 sums per cell and up to 65536 partials summed
+// by one warp 203 / 1449 / 79120; with this grid, link tables and FP64 sums
+// 55 / 215 / 9840; now 48 / 159 / 3945.
+template <class P, int DIMS, bool kQuads, int kLink, bool kDens>
 __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
   using C = typename P::cplx;
   using R = typename P::real;
-  const int x = blockIdx.x * 32 + threadIdx.x;
-  const int y = blockIdx.y * 8 + threadIdx.y;
+  constexpr int nc = nplanes<DIMS>() / 2;  // components, the lower ones from nc / 2
   const int Nx = a.N[0], Ny = a.N[1], Nz = DIMS == 3 ? a.N[2] : 1;
   const long long nxy = (long long)Nx * Ny;
+  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  const int tiles_x = (Nx + 31) / 32;
+  // rows summed: all of a whole grid, a slab's own levels zlo .. zlo + nzu - 1
+  // along the marching axis; fields at the global level
+  const int rows_y = DIMS == 3 ? Ny : a.nzu;
+  const long long items = (long long)tiles_x * rows_y * (DIMS == 3 ? a.nzu : 1);
   double acc[kObsSums] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  // (2+1)D: the summed rows zlo .. zlo + nzu - 1, fields at the global row
-  const bool row_in = DIMS == 3 || (y >= a.zlo && y < a.zlo + a.nzu);
-  int yg = y;
-  if (DIMS == 2) {
-    yg = a.zorg + y;  // in [-1, 2 Nzg): one wrap at most
-    if (yg < 0) yg += a.Nzg;
-    else if (yg >= a.Nzg) yg -= a.Nzg;
-  }
-  if (x < Nx && y < Ny && row_in) {
-    // the summed levels zlo .. zlo + nzu - 1; fields at their global level
-    for (int zz = blockIdx.z; zz < (DIMS == 3 ? a.nzu : 1); zz += gridDim.z) {
-      const int z = DIMS == 3 ? a.zlo + zz : 0;
-      int zg = DIMS == 3 ? a.zorg + z : 0;  // in [-1, 2 Nzg): one wrap at most
-      if (zg < 0) zg += a.Nzg;
-      else if (zg >= a.Nzg) zg -= a.Nzg;
-      const long long cell = z * nxy + (long long)y * Nx + x;
-      const int j[3] = {x, y, z};
-      const int Nn[3] = {Nx, Ny, Nz};
-      const long long stride[3] = {1, Nx, nxy};
-      R cn = 0, cd = 0, cb[3] = {0, 0, 0};
+  typename SumOf<P>::type sum[kObsSums] = {};
+  int pending = 0;
+  auto global_level = [&](int k) {  // in [-1, 2 Nzg): one wrap at most
+    const int g = a.zorg + k;
+    return g < 0 ? g + a.Nzg : (g >= a.Nzg ? g - a.Nzg : g);
+  };
+  for (long long it = (long long)blockIdx.x * wpb + (threadIdx.x >> 5); it < items; it += (long long)gridDim.x * wpb) {
+    const long long row = it / tiles_x;
+    const int x = (int)(it - row * tiles_x) * 32 + lane;
+    if (x >= Nx) continue;
+    const int zz = DIMS == 3 ? (int)(row / Ny) : 0;
+    const int y = DIMS == 3 ? (int)(row - (long long)zz * Ny) : a.zlo + (int)row;
+    const int z = DIMS == 3 ? a.zlo + zz : 0;
+    const int yg = DIMS == 3 ? y : global_level(y), zg = DIMS == 3 ? global_level(z) : 0;
+    const long long cell = z * nxy + (long long)y * Nx + x;
+    const long long dxm = x == 0 ? Nx - 1 : -1, dxp = x == Nx - 1 ? 1 - Nx : 1;
+    const long long dym = y == 0 ? nxy - Nx : -Nx, dyp = y == Ny - 1 ? Nx - nxy : Nx;
+    Pair<P> own[nc];
 #pragma unroll
-      for (int plane = 0; plane < nplanes<DIMS>(); ++plane) {
-        const C G = obs_value(a, plane, cell);
+    for (int c = 0; c < nc; ++c) own[c] = load_pair<P, kQuads>(a, c, cell);
+    R cn = 0, cd = 0, cb[3] = {0, 0, 0};
+#pragma unroll
+    for (int c = 0; c < nc; ++c) {
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        const C G = own[c].v[l];
         const R n2 = G.x * G.x + G.y * G.y;
         cn += n2;
-        long long H[3];
+        if (kDens) {
+          const int plane = 2 * c + l;
+          const int hd = a.dens_axis == 0 ? 2 * x + plane_off<DIMS>(plane, 0)
+                         : (a.dens_axis == 1 ? 2 * yg + plane_off<DIMS>(plane, 1) : 2 * zg + plane_off<DIMS>(plane, 2));
+          if (hd >= a.dens_X) cd += n2;
+        }
+      }
+    }
 #pragma unroll
-        for (int ax = 0; ax < 3; ++ax)
-          H[ax] = 2 * (ax == 2 ? zg : (ax == 1 ? yg : j[ax])) + plane_off<DIMS>(plane, ax);
-        const long long hd = a.dens_axis == 0 ? H[0] : (a.dens_axis == 1 ? H[1] : H[2]);
-        if (a.dens_axis >= 0 && hd >= a.dens_X) cd += n2;
-        if (is_upper<DIMS>(plane)) continue;
+    for (int c = nc / 2; c < nc; ++c) {
+      // the x-y partner component around the cell, the z partner above / below;
+      // sublattice 0 of C has its x+ neighbour in its own cell, of D (v) its x-
+      const int cxy = DIMS == 3 ? 3 - c : 0;
+      const bool kX = DIMS == 2 || c == 3;
+      const Pair<P> q = own[cxy];
+      const C xm = load_pair<P, kQuads>(a, cxy, cell + dxm).v[kX ? 1 : 0];
+      const C xp = load_pair<P, kQuads>(a, cxy, cell + dxp).v[kX ? 0 : 1];
+      const C ym1 = load_pair<P, kQuads>(a, cxy, cell + dym).v[1];
+      const C yp0 = load_pair<P, kQuads>(a, cxy, cell + dyp).v[0];
+      Pair<P> zu{}, zd{};
+      if (DIMS == 3) {
+        if (c == 2) {
+          zu = load_pair<P, kQuads>(a, 0, cell + (z == Nz - 1 ? nxy - nxy * Nz : nxy));
+          zd = own[0];
+        } else {
+          zu = own[1];
+          zd = load_pair<P, kQuads>(a, 1, cell + (z == 0 ? nxy * Nz - nxy : -nxy));
+        }
+      }
+      R wP[2], wQ[2];
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        const int plane = 2 * c + l;
+        const C G = own[c].v[l];
         const int p = sign_class<DIMS>(plane);
+        const long long H[3] = {2LL * x + plane_off<DIMS>(plane, 0), 2LL * yg + plane_off<DIMS>(plane, 1),
+                                DIMS == 3 ? 2LL * zg + plane_off<DIMS>(plane, 2) : 0};
 #pragma unroll
         for (int ax = 0; ax < DIMS; ++ax) {
-          const int pn = partner<DIMS>(plane, ax);
-          int jp = j[ax] + nb_shift<DIMS>(plane, ax, +1);
-          int jm = j[ax] + nb_shift<DIMS>(plane, ax, -1);
-          jp = jp >= Nn[ax] ? jp - Nn[ax] : jp;
-          jm = jm < 0 ? jm + Nn[ax] : jm;
-          C up = obs_value(a, pn, cell + (long long)(jp - j[ax]) * stride[ax]);
-          C dn = obs_value(a, pn, cell + (long long)(jm - j[ax]) * stride[ax]);
+          const bool own_up = (l == 0) != kX;  // the x+ neighbour is in the own cell
+          C up = ax == 0 ? (own_up ? q.v[l] : xp) : (ax == 1 ? (l == 0 ? q.v[1] : yp0) : zu.v[l]);
+          C dn = ax == 0 ? (own_up ? xm : q.v[l]) : (ax == 1 ? (l == 0 ? ym1 : q.v[0]) : zd.v[l]);
           R re, im;
-          if (a.link_mode == LINK_PLANE) {
-            // a plane wave with its wave vector across the polarisation (and no
-            // constant A on other axes): a phase on the polarisation axis only,
-            // the same for both links of the value (k has no component along them)
-            if (ax == a.f.Apw_pol) {
-              double sn, cs;
-              sincos(link_phase(a.f, DIMS, H, ax, +1, a.t_links), &sn, &cs);
-              const double2 u = widen(up), v = widen(dn);
-              // exp(-i phi) up - exp(+i phi) dn = cos phi (up - dn) - i sin phi (up + dn)
-              re = (R)(cs * (u.x - v.x) + sn * (u.y + v.y));
-              im = (R)(cs * (u.y - v.y) - sn * (u.x + v.x));
-            } else {
-              re = up.x - dn.x;
-              im = up.y - dn.y;
-            }
-          } else if (a.link_mode == LINK_GENERAL || a.link_mode == LINK_TABLE) {
-            double2 u = mul_expm(widen(up), link_phase_site(a.f, DIMS, H, ax, +1, a.t_links, plane, cell));
-            double2 v = mul_expm(widen(dn), -link_phase_site(a.f, DIMS, H, ax, -1, a.t_links, plane, cell));
+          if (kLink == LINK_PLANE && ax == a.f.Apw_pol) {  // (the wave is across its own links: one factor for both)
+            const R dr = up.x - dn.x, di = up.y - dn.y, qr = up.x + dn.x, qi = up.y + dn.y;
+            // s_a with s_x = 1; s_y = -i (p=0) / +i (p=1); s_z = +1 (p=0) / -1 (p=1),
+            // applied to both parts: conj(G) s_a (D) and conj(G) s_a (-i Q)
+            const R sdr = ax == 1 ? (p ? -di : di) : (ax == 2 && p ? -dr : dr);
+            const R sdi = ax == 1 ? (p ? dr : -dr) : (ax == 2 && p ? -di : di);
+            const R sqr = ax == 1 ? (p ? qr : -qr) : (ax == 2 && p ? -qi : qi);
+            const R sqi = ax == 1 ? (p ? qi : -qi) : (ax == 2 && p ? qr : -qr);
+            wP[l] = G.x * sdr + G.y * sdi;
+            wQ[l] = G.x * sqr + G.y * sqi;
+            continue;
+          } else if (kLink == LINK_GENERAL) {
+            const double2 u = mul_expm(widen(up), link_phase_site(a.f, DIMS, H, ax, +1, a.t_links, plane, cell));
+            const double2 v = mul_expm(widen(dn), -link_phase_site(a.f, DIMS, H, ax, -1, a.t_links, plane, cell));
             re = (R)(u.x - v.x);
             im = (R)(u.y - v.y);
           } else {
-            if (a.link_mode == LINK_CONST) {
+            if (kLink == LINK_CONST) {
               up = link_mul(a.L[ax], up);
               dn = link_mulc(a.L[ax], dn);
+            }
+            if constexpr (kLink == LINK_TABLE && kQuads) {
+              const float4* t = a.lq + 2 * ((long long)(2 * ax * nc + c) * a.pstride + cell);
+              const float4 u = quad_lane(t, l), d = quad_lane(t + 2 * nc * a.pstride, l);
+              up = link_mul(F32::Link{make_float2(u.x, u.y), make_float2(u.z, u.w)}, up);
+              dn = link_mulc(F32::Link{make_float2(d.x, d.y), make_float2(d.z, d.w)}, dn);
             }
             re = up.x - dn.x;
             im = up.y - dn.y;
           }
-          // s_a d: s_x = 1; s_y = -i (p=0) / +i (p=1); s_z = +1 (p=0) / -1 (p=1)
-          R sre = re, sim = im;
-          if (ax == 1) {
-            sre = p ? -im : im;
-            sim = p ? re : -re;
-          }
-          if (ax == 2 && p) {
-            sre = -re;
-            sim = -im;
-          }
+          const R sre = ax == 1 ? (p ? -im : im) : (ax == 2 && p ? -re : re);
+          const R sim = ax == 1 ? (p ? re : -re) : (ax == 2 && p ? -im : im);
           cb[ax] += G.x * sre + G.y * sim;  // Re(conj(G) s d)
         }
       }
-      acc[0] += (double)cn;
-      acc[1] += (double)cb[0];
-      acc[2] += (double)cb[1];
-      acc[3] += (double)cb[2];
-      acc[4] += (double)cd;
+      if (kLink == LINK_PLANE) {
+        const int k = a.wave_axis;
+        const int o0 = plane_off<DIMS>(2 * c, 0), o1 = plane_off<DIMS>(2 * c, 1);
+        // half-lattice coordinate along the wave vector of each value (along z both are at the same level)
+        const int h0 = k == 0 ? 2 * x + o0 : (k == 1 ? 2 * yg + o1 : 2 * zg + plane_off<DIMS>(2 * c, 2));
+        const int h1 = k == 0 ? 2 * x + 1 - o0 : (k == 1 ? 2 * yg + 1 - o1 : h0);
+        // the wave's terms go to its polarisation axis
+        auto wave_term = [&](int h, R pt, R qt) {
+#pragma unroll
+          for (int ax = 0; ax < DIMS; ++ax) {  // (an index known at compile time)
+            if (ax != a.f.Apw_pol) continue;
+            if constexpr (sizeof(R) == 4) {
+              const PlaneLink32* f = static_cast<const PlaneLink32*>(a.wave) + h;
+              sum[1 + ax].add_product(__ldg(&f->ch.x), __ldg(&f->cl.x), pt);
+              sum[1 + ax].add_product(__ldg(&f->sp.x), __ldg(&f->lp.x), qt);
+            } else {
+              const double2 f = __ldg(static_cast<const double2*>(a.wave) + h);  // (cos phi, -sin phi)
+              sum[1 + ax].add(f.x * pt - f.y * qt);
+            }
+          }
+        };
+        if (k == 2) {
+          wave_term(h0, wP[0] + wP[1], wQ[0] + wQ[1]);
+        } else {
+          wave_term(h0, wP[0], wQ[0]);
+          wave_term(h1, wP[1], wQ[1]);
+        }
+      }
+    }
+    sum[0].add(cn);
+#pragma unroll
+    for (int ax = 0; ax < DIMS; ++ax)
+      if (kLink != LINK_PLANE || ax != a.f.Apw_pol) sum[1 + ax].add(cb[ax]);
+    if (kDens) sum[4].add(cd);
+    if (++pending == kFlush) {
+      pending = 0;
+#pragma unroll
+      for (int k = 0; k < kObsSums; ++k) sum[k].flush(acc[k]);
     }
   }
-  const long long b = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  block_reduce_store<kObsSums>(acc, a.partials + b * kObsSums);
-}
-
-__global__ void finish_sums2_kernel(const double* partials, int nblocks, double* out) {
-  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
-  if (k >= 2) return;
-  double x = 0.0;
-  for (int b = lane; b < nblocks; b += 32) x += partials[2LL * b + k];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-  if (lane == 0) out[k] = x;
+  for (int k = 0; k < kObsSums; ++k) sum[k].flush(acc[k]);
+  block_reduce_store<kObsSums>(acc, a.partials + (long long)blockIdx.x * kObsSums);
 }
 
 // exp(-i phi) in the plane-wave table's element type: F64::Link, or for the
@@ -338,12 +436,19 @@ __global__ void link_factor_table_kernel(F32::Link* __restrict__ out, const Fiel
   }
 }
 
-__global__ void finish_sums_kernel(const double* partials, int nblocks, double* out) {
-  // warp k sums column k: lane-strided, then a fixed shuffle tree
+// out[k] = sum over the blocks of partials[block][k]: one warp per column,
+// eight loads in flight per lane, a fixed order
+template <int NS>
+__global__ void finish_sums_kernel(const double* __restrict__ partials, int nblocks, double* out) {
   const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
-  if (k >= kObsSums) return;
   double x = 0.0;
-  for (int b = lane; b < nblocks; b += 32) x += partials[(long long)b * kObsSums + k];
+  for (int b0 = lane; b0 < nblocks; b0 += 256) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = b0 + 32 * u < nblocks ? partials[(long long)(b0 + 32 * u) * NS + k] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x += v[u];
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
   if (lane == 0) out[k] = x;
@@ -445,25 +550,46 @@ double measure_fp64_fma_tflops() {
   return 2.0 * 8.0 * iters * (double)blocks * threads / (best * 1e-3) / 1e12;
 }
 
+// blocks of eight warps, a row piece of 32 cells per warp at a time: at most
+// four blocks on every SM (the launcher takes fewer where registers hold fewer)
 int observables_blocks(const int N[3], int dims) {
-  const int gx = (N[0] + 31) / 32, gy = (N[1] + 7) / 8;
-  const int nz = dims == 3 ? N[2] : 1;
-  long long per_z = (long long)gx * gy;
-  long long gz = (152LL * 8 + per_z - 1) / per_z;
-  if (gz > nz) gz = nz;
-  if (gz < 1) gz = 1;
-  return (int)(per_z * gz);
+  const long long items = (long long)((N[0] + 31) / 32) * N[1] * (dims == 3 ? N[2] : 1);
+  const long long b = (items + 7) / 8;
+  return (int)(b < 152 * 4 ? b : 152 * 4);
 }
 
-template <class P, int DIMS>
-void launch_observables(const ObsArgs<P>& a, int blocks, cudaStream_t s) {
-  const int gx = (a.N[0] + 31) / 32, gy = (a.N[1] + 7) / 8;
-  observables_kernel<P, DIMS><<<dim3(gx, gy, blocks / (gx * gy)), dim3(32, 8), 0, s>>>(a);
+template <class P, int DIMS, bool kQuads, int kLink, bool kDens>
+static int launch_observables_path(const ObsArgs<P>& a, int blocks, cudaStream_t s) {
+  constexpr auto k = observables_kernel<P, DIMS, kQuads, kLink, kDens>;
+  static const int resident = fused::resident_blocks(k, 256);  // a second, partial wave would idle most SMs
+  const int grid = blocks < resident ? blocks : resident;
+  k<<<grid, 256, 0, s>>>(a);
+  return grid;
 }
-template void launch_observables<F64, 2>(const ObsArgs<F64>&, int, cudaStream_t);
-template void launch_observables<F64, 3>(const ObsArgs<F64>&, int, cudaStream_t);
-template void launch_observables<F32, 2>(const ObsArgs<F32>&, int, cudaStream_t);
-template void launch_observables<F32, 3>(const ObsArgs<F32>&, int, cudaStream_t);
+template <class P, int DIMS, bool kQuads, bool kDens>
+static int launch_observables_link(const ObsArgs<P>& a, int blocks, cudaStream_t s) {
+  const int l = a.link_mode;
+  if (l == LINK_NONE) return launch_observables_path<P, DIMS, kQuads, LINK_NONE, kDens>(a, blocks, s);
+  if (l == LINK_CONST) return launch_observables_path<P, DIMS, kQuads, LINK_CONST, kDens>(a, blocks, s);
+  if (l == LINK_PLANE && a.wave) return launch_observables_path<P, DIMS, kQuads, LINK_PLANE, kDens>(a, blocks, s);
+  if (kQuads && l == LINK_TABLE)
+    return launch_observables_path<P, DIMS, kQuads, kQuads ? LINK_TABLE : LINK_GENERAL, kDens>(a, blocks, s);
+  return launch_observables_path<P, DIMS, kQuads, LINK_GENERAL, kDens>(a, blocks, s);
+}
+template <class P, int DIMS>
+int launch_observables(const ObsArgs<P>& a, int blocks, cudaStream_t s) {
+  if constexpr (sizeof(typename P::real) == 4) {
+    if (a.quads[0])
+      return a.dens_axis >= 0 ? launch_observables_link<P, DIMS, true, true>(a, blocks, s)
+                              : launch_observables_link<P, DIMS, true, false>(a, blocks, s);
+  }
+  return a.dens_axis >= 0 ? launch_observables_link<P, DIMS, false, true>(a, blocks, s)
+                          : launch_observables_link<P, DIMS, false, false>(a, blocks, s);
+}
+template int launch_observables<F64, 2>(const ObsArgs<F64>&, int, cudaStream_t);
+template int launch_observables<F64, 3>(const ObsArgs<F64>&, int, cudaStream_t);
+template int launch_observables<F32, 2>(const ObsArgs<F32>&, int, cudaStream_t);
+template int launch_observables<F32, 3>(const ObsArgs<F32>&, int, cudaStream_t);
 
 template <class P>
 void launch_link_table(void* tab, int n, const FieldDesc& f, int dims, int axis, int pol, double t_up,
@@ -522,11 +648,11 @@ void launch_link_factor_table(F32::Link* out, const FieldDesc& f, int dims, cons
 }
 
 void launch_finish_sums2(const double* partials, int nblocks, double* out, cudaStream_t s) {
-  finish_sums2_kernel<<<1, 64, 0, s>>>(partials, nblocks, out);
+  finish_sums_kernel<2><<<1, 64, 0, s>>>(partials, nblocks, out);
 }
 
 void launch_finish_sums(const double* partials, int nblocks, double* out, cudaStream_t s) {
-  finish_sums_kernel<<<1, 32 * kObsSums, 0, s>>>(partials, nblocks, out);
+  finish_sums_kernel<kObsSums><<<1, 32 * kObsSums, 0, s>>>(partials, nblocks, out);
 }
 
 static unsigned grid_for(long long n) {
