@@ -359,9 +359,10 @@ double dirac_algorithmic_bytes(const dirac_sim* sim);
 /* device bytes a simulation of this shape and precision allocates for a
    potential made of V0 and a Klein step only: the state, plus for
    DIRAC_FP32 a second state buffer and one complex128 conversion plane.
-   Other potentials add one double per value (DIRAC_FP64, or a time-
-   dependent static array) or the coefficient table, 16 bytes per value
-   (DIRAC_FP32, time-independent), A_links 16 bytes per axis and value, a
+   Other potentials add one double per value (a static array that DIRAC_FP64
+   or a time dependence keeps) and the coefficient table, 16 bytes per value
+   (DIRAC_FP32, time-independent) or 32 (DIRAC_FP64, time-independent, where
+   that leaves at least as much device memory free), A_links 16 bytes per axis and value, a
    tabulated static vector potential (DIRAC_FP32) 32 bytes per axis and
    value, and every simulation a few KiB of reduction scratch. */
 size_t dirac_state_bytes(int dims, const int N[3], dirac_precision precision);

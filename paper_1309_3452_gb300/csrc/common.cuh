@@ -265,7 +265,9 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // COEF_TABLE: a time-independent scalar potential (soft core, static array,
 // with V0 and a Klein step) whose coefficient b = 1/(1 + i theta), theta =
 // dt (beta m + V)/2, is tabulated per site at creation, in FP64 rounded to a
-// hi + lo pair of complex floats (FP32 kernels).  LINK_PLANE: a plane-wave vector potential whose wave vector lies
+// hi + lo pair of complex floats (FP32 kernels), or as alpha and gamma in FP64
+// (FP64 kernels, whose FP64 pipe a square root and a division per value and
+// half-step would keep 10 times longer than the update itself).  LINK_PLANE: a plane-wave vector potential whose wave vector lies
 // along one axis other than its polarisation; its link factors come from a
 // per-half-step table indexed by the half-lattice coordinate along that axis.
 // LINK_TABLE: any other time-independent vector potential (FP32 kernels): the
@@ -359,6 +361,16 @@ __device__ __forceinline__ double potential_at(const FieldDesc& f, int dims, lon
   }
   if (f.Vstatic) V += f.Vstatic[(long long)plane * pstride + site] * (1.0 + f.Vmod_amp * cos(f.Vmod_omega * t));
   return V;
+}
+
+// alpha and gamma of the value at half-lattice point (X, Y, Z) at time t
+__device__ __forceinline__ void site_coef(const FieldDesc& f, int dims, long long X, long long Y, long long Z,
+                                          long long site, long long pstride, int plane, double beta, double t,
+                                          double2& al, double2& ga) {
+  const double V = potential_at(f, dims, X, Y, Z, site, pstride, plane, t);
+  const double th = f.dt * (beta * f.m + V) * 0.5;
+  const double th_im = f.dt * potential_imag_at(f, dims, X, Y, Z) * 0.5;
+  coef_from_theta(th, th_im, f.rx, al, ga);
 }
 
 // link phase phi = q * (line integral of A_a along the link, Sect. 4) for the
@@ -563,7 +575,10 @@ struct HalfFields {
   double beta;              // +1 upper (A,B,u), -1 lower (C,D,v)
   // COEF_TABLE: b of every site as {re hi, im hi, re lo, im lo}, one array
   // per plane (cell index as in the state), and r_x as hi + lo
+  // (FP64 kernels: alpha and gamma of every site, c_tab + plane * c_ps + cell)
   const float4* b_tab[8];
+  const typename P::Coef* c_tab;
+  long long c_ps;
   float rx_hi, rx_lo;
   // LINK_PLANE: table of the link factors exp(-i phi) for this half-step,
   // indexed by the half-lattice coordinate along ltab_axis; applies on axis
@@ -616,8 +631,9 @@ __device__ __forceinline__ F32::Link table_link(const HalfFields<F32>& h, int sl
   return h.larr[slot * h.larr_n + (long long)plane * h.larr_ps + site];
 }
 
-// The tabulated-potential update (F32 only), the paper's form of the Cayley
-// step (Eqs. ss1-ss4):  F+ = b (2F - S) - F,  b = 1/(1 + i theta),  S = r_x S'
+// The tabulated-potential update.  FP64: alpha F - gamma S' with the site's own
+// alpha and gamma, formed once by the operations of the per-site path (same
+// bits).  F32: the paper's form of the Cayley step (Eqs. ss1-ss4):  F+ = b (2F - S) - F,  b = 1/(1 + i theta),  S = r_x S'
 // which is ((1 - i theta) F - S)/(1 + i theta).  b and r_x are carried as
 // hi + lo pairs, so |2b - 1| = 1 holds to ~1e-14 and the rounding of the
 // coefficients does not accumulate over steps.
@@ -625,9 +641,10 @@ template <class P>
 __device__ __forceinline__ typename P::cplx apply_table(const HalfFields<P>& h, typename P::cplx F,
                                                         typename P::cplx S, int plane, long long site);
 template <>
-__device__ __forceinline__ double2 apply_table<F64>(const HalfFields<F64>&, double2 F, double2, int,
-                                                    long long) {
-  return F;  // not used: FP64 kernels take the general path
+__device__ __forceinline__ double2 apply_table<F64>(const HalfFields<F64>& h, double2 F, double2 S, int plane,
+                                                    long long site) {
+  const double2* c = reinterpret_cast<const double2*>(h.c_tab + (plane * h.c_ps + site));
+  return apply(F64::Coef{__ldg(c), __ldg(c + 1)}, F, S);
 }
 template <>
 __device__ __forceinline__ float2 apply_table<F32>(const HalfFields<F32>& h, float2 F, float2 S, int plane,
@@ -790,11 +807,8 @@ __device__ __forceinline__ typename P::cplx site_update(
     if constexpr (sizeof(typename P::real) == 4) return apply_softcorr_f32<DIMS>(h, F, S, H, plane, Ngrid);
     else return F;  // not used: FP64 kernels take the general path
   }
-  double V = potential_at(f, DIMS, H[0], H[1], H[2], site, pstride, plane, h.t);
-  double th = f.dt * (h.beta * f.m + V) * 0.5;
-  double th_im = f.dt * potential_imag_at(f, DIMS, H[0], H[1], H[2]) * 0.5;
   double2 al, ga;
-  coef_from_theta(th, th_im, f.rx, al, ga);
+  site_coef(f, DIMS, H[0], H[1], H[2], site, pstride, plane, h.beta, h.t, al, ga);
   return apply(coef_from(al, ga, (P*)nullptr), F, S);
 }
 

@@ -43,8 +43,10 @@ struct dirac_sim {
   double plan_us = 0;         // time per step the autotuner measured for the plan
   double2* staging = nullptr; // one canonical plane (FP32 conversions)
   double* Vstatic = nullptr;  // one real per site (plane-major, pstride)
+  int vstatic = 0;            // the caller gave a static array (which a table may have replaced)
   float4* b_tab = nullptr;    // COEF_TABLE: b = 1/(1 + i theta) per site as hi + lo (plane-major, pstride)
   float2* sc_sq = nullptr;    // COEF_SOFTCORE/CORR: (X dx_a/2 - c_a)^2 per axis and half-lattice index, hi + lo
+  F64::Coef* c_tab = nullptr; // COEF_TABLE, FP64: alpha and gamma per site (plane-major, pstride)
   unsigned* sc_corr = nullptr; // COEF_SOFTCORR: one 32-bit correction word per value
   double* Alink = nullptr;    // link integrals x q: 2 dims slots (up, down link per axis) of np * pstride
   F32::Link* larr = nullptr;  // LINK_TABLE: link factors, same slots, FP32 hi + lo
@@ -297,6 +299,8 @@ static HalfFields<P> half_fields(const dirac_sim* s, bool upper, double t) {
   // tabulated potential
   for (int k = 0; k < 8; ++k)
     h.b_tab[k] = s->b_tab && !s->fused && k < s->np ? s->b_tab + (long long)k * s->pstride : nullptr;
+  h.c_tab = reinterpret_cast<const typename P::Coef*>(s->c_tab);
+  h.c_ps = s->pstride;
   if (s->fused) {
     h.bq = s->b_tab;
     h.lq = s->link_mode == LINK_TABLE ? reinterpret_cast<const float4*>(s->larr) : nullptr;
@@ -527,6 +531,7 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
   // a time-independent potential beyond V0 and the step: tabulated for the FP32
   // kernels, evaluated per site in FP64 otherwise
   const bool vstatic = fields && fields->V_static;
+  s->vstatic = vstatic;
   const bool layers = f.abs_W != 0.0;
   // a real soft core (with V0 and a Klein step, nothing else): analytic per
   // value in the FP32 kernels, no per-site data
@@ -664,7 +669,28 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
       s->coef_mode = COEF_SOFTCORE;
     }
   }
-  if (s->coef_mode == COEF_TABLE) {
+  if (s->coef_mode == COEF_GENERAL && !(s->Vstatic && f.Vmod_amp != 0.0)) {
+    // FP64, a potential that does not change in time: tabulated where the table
+    // leaves the caller as much free device memory as it takes, else evaluated
+    // per site (same values)
+    const size_t tb = (size_t)s->np * s->pstride * sizeof(F64::Coef);
+    size_t mem_free = 0, mem_total = 0;
+    if ((e = cudaMemGetInfo(&mem_free, &mem_total)) != cudaSuccess)
+      return cleanup_fail(cuda_fail(s, e, "cudaMemGetInfo"));
+    e = tb <= mem_free / 2 ? cudaMalloc(&s->c_tab, tb) : cudaErrorMemoryAllocation;
+    if (e == cudaSuccess) {
+      launch_coef64_table(s->c_tab, field_desc(s), dims, s->N, s->pstride, s->stream);
+      if ((e = cudaGetLastError()) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "coefficient table"));
+      s->launches += 1;
+      s->coef_mode = COEF_TABLE;
+    } else if (e == cudaErrorMemoryAllocation) {
+      s->c_tab = nullptr;
+      cudaGetLastError();  // not an error of this simulation
+    } else {
+      return cleanup_fail(cuda_fail(s, e, "cudaMalloc(coefficient table)"));
+    }
+  }
+  if (s->coef_mode == COEF_TABLE && !s->c_tab) {
     if ((e = cudaMalloc(&s->b_tab, (size_t)s->np * s->pstride * sizeof(float4))) != cudaSuccess)
       return cleanup_fail(cuda_fail(s, e, "cudaMalloc(coefficient table)"));
     launch_coef_table(s->b_tab, field_desc(s), dims, s->N, s->pstride, s->fused, s->stream);
@@ -719,6 +745,7 @@ extern "C" void dirac_destroy(dirac_sim* s) {
   cudaFree(s->staging);
   cudaFree(s->Vstatic);
   cudaFree(s->b_tab);
+  cudaFree(s->c_tab);
   cudaFree(s->sc_sq);
   cudaFree(s->sc_corr);
   cudaFree(s->Alink);
@@ -1613,9 +1640,11 @@ extern "C" dirac_status dirac_check(dirac_sim* s, double tol, dirac_check_report
 extern "C" double dirac_algorithmic_bytes(const dirac_sim* s) {
   if (!s) return 0.0;
   double b = 2.0 * s->np * (double)s->elem;                    // every value read and written once
-  if (s->coef_mode == COEF_TABLE) b += 16.0 * s->np;           // one coefficient per value read
+  // one coefficient per value read (FP64's table of alpha and gamma is the
+  // library's choice: there the data given per site counts, below)
+  if (s->coef_mode == COEF_TABLE && !s->c_tab) b += 16.0 * s->np;
   if (s->coef_mode == COEF_SOFTCORR) b += 4.0 * s->np;         // one correction word per value read
-  if (s->coef_mode == COEF_GENERAL && s->Vstatic) b += 8.0 * s->np;  // one real per value read
+  if ((s->coef_mode == COEF_GENERAL && s->Vstatic) || (s->c_tab && s->vstatic)) b += 8.0 * s->np;  // one real per value
   if (s->link_mode == LINK_TABLE) b += 32.0 * s->dims * s->np;  // up and down link factor (hi + lo) per axis
   else if (s->Alink) b += 16.0 * s->dims * s->np;              // up and down link integral per axis
   return b;

@@ -138,6 +138,10 @@ void launch_link_table(void* tab, int n, const FieldDesc& f, int dims, int axis,
 void launch_coef_table(float4* tab, const FieldDesc& f, int dims, const int N[3], long long pstride, int quads,
                        cudaStream_t s);
 
+// the FP64 kernels' table: alpha and gamma of every value, tab[plane * pstride + cell]
+void launch_coef64_table(F64::Coef* tab, const FieldDesc& f, int dims, const int N[3], long long pstride,
+                         cudaStream_t s);
+
 // COEF_SOFTCORR correction records of a soft-core potential (one 32-bit word
 // per value, softcore_corr_index's layout); *overflow (device) is or-ed with 1
 // if a correction does not fit

@@ -340,6 +340,25 @@ __global__ void coef_table_kernel(float4* __restrict__ tab, const FieldDesc f, i
   }
 }
 
+// COEF_TABLE of the FP64 kernels: alpha and gamma of every site, by the same
+// operations as the per-site path
+template <int DIMS>
+__global__ void coef64_table_kernel(F64::Coef* __restrict__ tab, const FieldDesc f, int N0, int N1, int N2,
+                                    long long pstride) {
+  const int plane = blockIdx.y;
+  const long long ncell = (long long)N0 * N1 * N2;
+  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
+       c += (long long)gridDim.x * blockDim.x) {
+    const long long x = c % N0, y = (c / N0) % N1, z = c / ((long long)N0 * N1);
+    const long long X = 2 * x + plane_off<DIMS>(plane, 0), Y = 2 * y + plane_off<DIMS>(plane, 1),
+                    Z = DIMS == 3 ? 2 * z + plane_off<DIMS>(plane, 2) : 0;
+    const double beta = is_upper<DIMS>(plane) ? 1.0 : -1.0;
+    double2 al, ga;
+    site_coef(f, DIMS, X, Y, Z, c, pstride, plane, beta, 0.0, al, ga);
+    tab[plane * pstride + c] = F64::Coef{al, ga};
+  }
+}
+
 // COEF_SOFTCORR: the correction records (softcore_corr_index's layout) of a
 // real soft-core potential: per value, (exact b) - (the kernels' FP32
 // estimate softcore_fast2), b = 1/(1 + i dt (beta m + V)/2) with V from the
@@ -610,6 +629,18 @@ void launch_coef_table(float4* tab, const FieldDesc& f, int dims, const int N[3]
     coef_table_kernel<3><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], N[2], pstride, quads);
   else
     coef_table_kernel<2><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], 1, pstride, quads);
+}
+
+void launch_coef64_table(F64::Coef* tab, const FieldDesc& f, int dims, const int N[3], long long pstride,
+                         cudaStream_t s) {
+  const long long ncell = (long long)N[0] * N[1] * (dims == 3 ? N[2] : 1);
+  long long bx = (ncell + 255) / 256;
+  if (bx > 152 * 16) bx = 152 * 16;
+  const dim3 grid((unsigned)bx, dims == 3 ? 8 : 4);
+  if (dims == 3)
+    coef64_table_kernel<3><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], N[2], pstride);
+  else
+    coef64_table_kernel<2><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], 1, pstride);
 }
 
 void launch_softcore_corr(unsigned* out, const HalfFields<F32>& hu, const HalfFields<F32>& hl, const FieldDesc& f,

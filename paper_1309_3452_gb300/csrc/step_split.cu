@@ -54,28 +54,23 @@ void launch_one(const HalfStepArgs<P>& a, cudaStream_t s) {
   dim3 grid((a.N[0] + 31) / 32, (a.N[1] + 3) / 4, DIMS == 3 ? a.N[2] : 1);
   const int c = a.h.coef_mode, l = a.h.link_mode;
   constexpr bool f32 = sizeof(typename P::real) == 4;
-  if (c == COEF_UNIFORM && l == LINK_NONE)
-    half_step_kernel<P, DIMS, UPPER, COEF_UNIFORM, LINK_NONE><<<grid, block, 0, s>>>(a);
-  else if (c == COEF_STEP && l == LINK_NONE)
-    half_step_kernel<P, DIMS, UPPER, COEF_STEP, LINK_NONE><<<grid, block, 0, s>>>(a);
-  else if (f32 && c == COEF_TABLE && l == LINK_NONE)  // the FP32 tabulated-potential paths
-    half_step_kernel<P, DIMS, UPPER, COEF_TABLE, LINK_NONE><<<grid, block, 0, s>>>(a);
-  else if (f32 && c == COEF_SOFTCORE && l == LINK_NONE)  // the FP32 analytic soft core
-    half_step_kernel<P, DIMS, UPPER, COEF_SOFTCORE, LINK_NONE><<<grid, block, 0, s>>>(a);
-  else if (f32 && c == COEF_SOFTCORE && l == LINK_PLANE)
-    half_step_kernel<P, DIMS, UPPER, COEF_SOFTCORE, LINK_PLANE><<<grid, block, 0, s>>>(a);
-  else if (f32 && c == COEF_SOFTCORR && l == LINK_NONE)
-    half_step_kernel<P, DIMS, UPPER, COEF_SOFTCORR, LINK_NONE><<<grid, block, 0, s>>>(a);
-  else if (f32 && c == COEF_SOFTCORR && l == LINK_PLANE)
-    half_step_kernel<P, DIMS, UPPER, COEF_SOFTCORR, LINK_PLANE><<<grid, block, 0, s>>>(a);
-  else if (f32 && c == COEF_TABLE && l == LINK_PLANE)
-    half_step_kernel<P, DIMS, UPPER, COEF_TABLE, LINK_PLANE><<<grid, block, 0, s>>>(a);
-  else if (f32 && c == COEF_UNIFORM && l == LINK_PLANE)
-    half_step_kernel<P, DIMS, UPPER, COEF_UNIFORM, LINK_PLANE><<<grid, block, 0, s>>>(a);
-  else if (f32 && c == COEF_STEP && l == LINK_PLANE)
-    half_step_kernel<P, DIMS, UPPER, COEF_STEP, LINK_PLANE><<<grid, block, 0, s>>>(a);
-  else
-    half_step_kernel<P, DIMS, UPPER, kAnyMode, kAnyMode><<<grid, block, 0, s>>>(a);
+#define HALF_STEP(COEF, LINK) half_step_kernel<P, DIMS, UPPER, COEF, LINK><<<grid, block, 0, s>>>(a)
+  if (c == COEF_UNIFORM && l == LINK_NONE) HALF_STEP(COEF_UNIFORM, LINK_NONE);
+  else if (c == COEF_STEP && l == LINK_NONE) HALF_STEP(COEF_STEP, LINK_NONE);
+  else if (c == COEF_TABLE && l == LINK_NONE) HALF_STEP(COEF_TABLE, LINK_NONE);
+  else if (c == COEF_UNIFORM && l == LINK_PLANE) HALF_STEP(COEF_UNIFORM, LINK_PLANE);
+  else if (c == COEF_STEP && l == LINK_PLANE) HALF_STEP(COEF_STEP, LINK_PLANE);
+  else if (c == COEF_TABLE && l == LINK_PLANE) HALF_STEP(COEF_TABLE, LINK_PLANE);
+  else if (f32 && c == COEF_SOFTCORE && l == LINK_NONE) HALF_STEP(f32 ? COEF_SOFTCORE : COEF_TABLE, LINK_NONE);
+  else if (f32 && c == COEF_SOFTCORE && l == LINK_PLANE) HALF_STEP(f32 ? COEF_SOFTCORE : COEF_TABLE, LINK_PLANE);
+  else if (f32 && c == COEF_SOFTCORR && l == LINK_NONE) HALF_STEP(f32 ? COEF_SOFTCORR : COEF_TABLE, LINK_NONE);
+  else if (f32 && c == COEF_SOFTCORR && l == LINK_PLANE) HALF_STEP(f32 ? COEF_SOFTCORR : COEF_TABLE, LINK_PLANE);
+  // FP64 (the FP32 reference kernels take these through the run-time path)
+  else if (!f32 && c == COEF_UNIFORM && l == LINK_CONST) HALF_STEP(COEF_UNIFORM, f32 ? LINK_NONE : LINK_CONST);
+  else if (!f32 && c == COEF_STEP && l == LINK_CONST) HALF_STEP(COEF_STEP, f32 ? LINK_NONE : LINK_CONST);
+  else if (!f32 && c == COEF_TABLE && l == LINK_CONST) HALF_STEP(COEF_TABLE, f32 ? LINK_NONE : LINK_CONST);
+  else HALF_STEP(kAnyMode, kAnyMode);
+#undef HALF_STEP
 }
 
 }  // namespace
