@@ -87,8 +87,10 @@ struct F32 {
 // table (c = c_hi + c_lo, s = s_hi + s_lo), kept as the packed operand pairs
 // of plane_link_diff: ch = (c_hi, c_hi), cl = (c_lo, c_lo), sh = (s_hi, -s_hi),
 // sl = (s_lo, -s_lo) (one value: lanes re, im) and sp = (s_hi, s_hi), lp =
-// (s_lo, s_lo) (two values: lanes are the two sublattices, quad.cuh)
+// (s_lo, s_lo) (two values: lanes are the two sublattices, quad.cuh); v =
+// (c_hi, c_lo, s_hi, s_lo) for lanes with factors of their own
 struct PlaneLink32 {
+  float4 v;
   float2 ch, cl, sh, sl, sp, lp;
 };
 
@@ -260,6 +262,9 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the newest kN groups of the issuing thread have landed
+template <int kN>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kN) : "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // COEF_TABLE: a time-independent scalar potential (soft core, static array,
@@ -287,6 +292,13 @@ enum LinkMode { LINK_NONE = 0, LINK_CONST = 1, LINK_GENERAL = 2, LINK_PLANE = 3,
 // wave travels along z and is polarised along x; the kernel stages the link
 // factors of each z level and passes them in (never a simulation's link_mode)
 constexpr int LINK_PLANE_ZX = 5;
+// Kernel-side specialisation of COEF_STEP: every value of the work lies beyond the step
+constexpr int COEF_BEYOND = 6;
+// ... or the step lies between the lanes of a warp: each lane's coefficients
+// are in shared memory (quad.cuh, lane_coefs)
+constexpr int COEF_LANES = 7;
+// Kernel-side specialisation of COEF_STEP in (2+1)D: the step is across x
+constexpr int COEF_STEP_X = 8;
 
 // Analytic field description, FP64, for the per-site (general) paths.
 struct FieldDesc {

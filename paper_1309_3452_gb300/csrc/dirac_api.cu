@@ -38,8 +38,8 @@ struct dirac_sim {
   void* state_alt = nullptr;  // second buffer for the out-of-place fused kernels
   int fused = 0;              // one kernel per time step (FP32 without the reference flag); the state
                               // (and the per-site tables) are then held as quads (quad.cuh)
-  int tblock = 1;             // (2+1)D fused path: two time steps per pass when possible
-  int chunk1 = 0, chunk2 = 0; // launch plan: levels per item (one-step / two-step kernel), 0 = rule
+  int tblock = 1;             // (2+1)D fused path: several time steps per pass when possible
+  int chunk1 = 0, chunk2 = 0; // launch plan: levels per item (passes of one / several steps), 0 = rule
   double plan_us = 0;         // time per step the autotuner measured for the plan
   double2* staging = nullptr; // one canonical plane (FP32 conversions)
   double* Vstatic = nullptr;  // one real per site (plane-major, pstride)
@@ -69,6 +69,7 @@ struct dirac_sim {
   // (only for fields without time dependence: the launches bake their time)
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   void* graph_state[2] = {nullptr, nullptr};
+  long long graph_launches[2] = {0, 0};  // kernels in each
   int graph_disabled = 0;
   int stepped = 0;            // a plain step has run (kernel one-time set-up done)
   // conserved functional accumulated by the last fused launch of a dirac_step
@@ -374,6 +375,7 @@ static FusedArgs<P> fused_args(dirac_sim* s, double t) {
   a.rz = make_ratio<P>((s->dt / s->dx[2]) / rx);
   a.hu = half_fields<P>(s, true, t);
   a.hl = half_fields<P>(s, false, t + s->dt / 2.0);
+  a.lstep = s->link_mode == LINK_PLANE ? 2 * s->ltab_n : 0;
   a.f = field_desc(s);
   a.zlo = s->zlo;
   a.nzu = s->nzu;
@@ -517,7 +519,7 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
     s->nzu = slab.nz;
     s->zorg = slab.z0 - 1;
     s->Nzg = slab.Nzg;
-    s->tblock = 0;  // two-step passes would need two halo levels
+    s->tblock = 0;  // passes of several steps would need as many halo levels
   } else {
     s->zlo = 0;
     s->nzu = s->Nzg = s->N[march];
@@ -698,8 +700,9 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
     s->launches += 1;
   }
   if (s->link_mode == LINK_PLANE) {
-    size_t tb = (size_t)2 * s->ltab_n * (precision == DIRAC_FP32 ? sizeof(PlaneLinkOf<F32>::type)
-                                                                 : sizeof(PlaneLinkOf<F64>::type));
+    // (a pass of several (2+1)D steps has a table per step)
+    size_t tb = (size_t)2 * (dims == 2 ? kMaxSteps2d : 1) * s->ltab_n *
+                (precision == DIRAC_FP32 ? sizeof(PlaneLinkOf<F32>::type) : sizeof(PlaneLinkOf<F64>::type));
     if ((e = cudaMalloc(&s->ltab, tb)) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link table)"));
     if ((e = cudaMalloc(&s->wave, tb)) != cudaSuccess)
       return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link table)"));
@@ -937,12 +940,18 @@ static bool time_dependent_fields(const dirac_sim* s) {
   return (s->Vstatic && s->f.Vmod_amp != 0.0) || moving_vector_potential(s);
 }
 
-// LINK_PLANE: tabulate this step's link factors (both half-steps)
+static double time_after(const dirac_sim* s, long long steps) { return s->t0 + (double)(s->k + steps) * s->dt; }
+
+// LINK_PLANE: tabulate the link factors of the next `steps` steps (both half-steps)
 template <class P>
-static void link_table(dirac_sim* s, double t, cudaStream_t st) {
+static void link_table(dirac_sim* s, int steps, cudaStream_t st) {
   if (s->link_mode != LINK_PLANE) return;
-  launch_link_table<P>(s->ltab, s->ltab_n, field_desc(s), s->dims, s->ltab_axis, s->f.Apw_pol, t,
-                       t + s->dt / 2.0, st);
+  double up[kMaxSteps2d], lo[kMaxSteps2d];
+  for (int j = 0; j < steps; ++j) {
+    up[j] = time_after(s, j);
+    lo[j] = up[j] + s->dt / 2.0;
+  }
+  launch_link_table<P>(s->ltab, s->ltab_n, field_desc(s), s->dims, s->ltab_axis, s->f.Apw_pol, up, lo, steps, st);
   s->launches += 1;
 }
 
@@ -950,7 +959,7 @@ template <class P>
 static dirac_status steps_split(dirac_sim* s, long n, cudaStream_t st) {
   for (long i = 0; i < n; ++i) {
     double t = sim_time(s);
-    link_table<P>(s, t, st);
+    link_table<P>(s, 1, st);
     HalfStepArgs<P> up = half_args<P>(s, true, t);
     HalfStepArgs<P> lo = half_args<P>(s, false, t + s->dt / 2.0);
     if (s->dims == 3) {
@@ -967,41 +976,46 @@ static dirac_status steps_split(dirac_sim* s, long n, cudaStream_t st) {
   return DIRAC_OK;
 }
 
+// the fused kernels run these field paths per site (run-time paths in FP64)
+static bool per_site_path(const dirac_sim* s) {
+  const int c = s->coef_mode, l = s->link_mode;
+  if (c == COEF_GENERAL || l == LINK_GENERAL) return true;
+  if (c == COEF_SOFTCORE || c == COEF_SOFTCORR) return l == LINK_CONST || l == LINK_TABLE;
+  return c == COEF_TABLE && l == LINK_CONST;
+}
+
+// Time steps per pass for the next n steps: (2+1)D whole grids take two where
+// the field path is not per site (a plane wave may move: its passes have a
+// table per step); the grid needs four rows.
+static int steps_per_pass(const dirac_sim* s, long n) {
+  const bool whole = s->zlo == 0 && s->zorg == 0 && s->nzu == s->Nzg;
+  if (s->dims != 2 || !s->tblock || !whole || per_site_path(s) ||
+      std::getenv("DIRAC_NO_TEMPORAL_BLOCKING") != nullptr)
+    return 1;
+  return n >= 2 && s->N[1] >= 4 ? 2 : 1;
+}
+
 // want_e: the last launch also accumulates the conserved functional of the
 // new state (dirac_norm then needs no reduction pass over the state)
 template <class P>
 static dirac_status steps_fused(dirac_sim* s, long n, cudaStream_t st, bool want_e) {
   want_e = want_e && n > 0 && std::getenv("DIRAC_NO_FUSED_NORM") == nullptr;
   int e_blocks = 0;
-  // (2+1)D, time-independent fields: two steps per pass while pairs remain
-  // (the two-step kernel takes whole grids: never a slab of a decomposed one)
-  const bool whole = s->zlo == 0 && s->zorg == 0 && s->nzu == s->Nzg;
-  const bool tb = s->dims == 2 && s->tblock && whole && !time_dependent_fields(s) &&
-                  std::getenv("DIRAC_NO_TEMPORAL_BLOCKING") == nullptr;
-  while (tb && n >= 2) {
+  while (n > 0) {
+    const int steps = steps_per_pass(s, n);
+    link_table<P>(s, steps, st);
     FusedArgs<P> a = fused_args<P>(s, sim_time(s));
-    a.chunk = s->chunk2;
-    if (want_e && n == 2) a.e_partials = s->e_partials;
-    const int blocks = launch_fused2d_tb2(a, st);
-    if (!blocks) break;
+    a.chunk = steps > 1 ? s->chunk2 : s->chunk1;
+    if (want_e && n == steps) a.e_partials = s->e_partials;
+    const int blocks = steps > 1 ? launch_fused2d_two(a, st)
+                                 : (s->dims == 3 ? launch_fused<P, 3>(a, st) : launch_fused<P, 2>(a, st));
+    if (!blocks) return fail(s, DIRAC_ERR_UNSUPPORTED, "no kernel of several steps for these fields");
     if (a.e_partials) e_blocks = blocks;
     s->launches += 1;
     CK(s, cudaGetLastError());
     std::swap(s->state, s->state_alt);
-    s->k += 2;
-    n -= 2;
-  }
-  for (long i = 0; i < n; ++i) {
-    link_table<P>(s, sim_time(s), st);
-    FusedArgs<P> a = fused_args<P>(s, sim_time(s));
-    a.chunk = s->chunk1;
-    if (want_e && i == n - 1) a.e_partials = s->e_partials;
-    const int blocks = s->dims == 3 ? launch_fused<P, 3>(a, st) : launch_fused<P, 2>(a, st);
-    if (a.e_partials) e_blocks = blocks;
-    s->launches += 1;
-    CK(s, cudaGetLastError());
-    std::swap(s->state, s->state_alt);
-    s->k += 1;
+    s->k += steps;
+    n -= steps;
   }
   if (e_blocks > 0 && e_blocks <= kFusedEMaxBlocks) {
     launch_finish_sums2(s->e_partials, e_blocks, s->e_sums, st);
@@ -1035,6 +1049,7 @@ static dirac_status build_graph(dirac_sim* s, int slot) {
     e = cudaStreamEndCapture(cap, &g);
   }
   // capturing did not run anything: restore the bookkeeping
+  s->graph_launches[slot] = s->launches - l0;
   s->k = k0;
   s->launches = l0;
   if (s->state != state0) std::swap(s->state, s->state_alt);
@@ -1078,9 +1093,9 @@ extern "C" dirac_status dirac_step(dirac_sim* s, long nsteps) {
       if (s->graph_disabled) break;
     }
     CK(s, cudaGraphLaunch(s->graph[slot], s->stream));
-    s->launches += kGraphSteps * (s->fused ? 1 : 2);
+    s->launches += s->graph_launches[slot];
     s->k += kGraphSteps;
-    if (s->fused && (kGraphSteps & 1)) std::swap(s->state, s->state_alt);
+    if (s->fused && (s->graph_launches[slot] & 1)) std::swap(s->state, s->state_alt);
     nsteps -= kGraphSteps;
   }
   return steps_plain(s, nsteps, s->stream, true);
@@ -1102,7 +1117,7 @@ struct BatchGraph {
   std::vector<void*> states;
   std::vector<int> chunks;
   long nsteps = 0;
-  int tb = 0;
+  int deepest = 0;
   void* tables = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaStream_t stream = nullptr;  // the group's stream, where the graph runs
@@ -1136,46 +1151,61 @@ static void drop_batch_graphs(const dirac_sim* s) {
   }
 }
 
-// the launches of one batched call: pairs of steps (two-step kernel) first,
-// then single steps; every launch swaps the buffers
-static cudaError_t enqueue_batch(const FusedArgs<F32>* d_args, const long long* first, int n, long pairs,
-                                 long launches, long long total, long long total2, int dims, int coef,
-                                 int link, cudaStream_t st) {
+// Launch modes of a batched call: passes of one and two steps (mode m: m + 1)
+static const int kBatchModes = 2;
+struct BatchPasses {
+  long count[kBatchModes] = {0, 0};       // launches of each mode; passes of two run first
+  long long items[kBatchModes] = {0, 0};  // work items of the group
+  long launches() const { return count[0] + count[1]; }
+};
+
+// every launch swaps the buffers; argument tables [mode][buffer parity][sim],
+// item prefix sums [mode][n + 1]
+static cudaError_t enqueue_batch(const FusedArgs<F32>* d_args, const long long* first, int n, const BatchPasses& p,
+                                 int dims, int coef, int link, bool iso, cudaStream_t st) {
   BatchArgs<F32> b;
   b.nsims = n;
   b.workers = 0;
-  for (long i = 0; i < launches; ++i) {
-    b.sims = d_args + ((i < pairs ? 2 : 0) + (i & 1)) * n;
-    if (i < pairs) {
-      b.first_item = first + n + 1;
-      launch_fused2d_tb2_batch(b, total2, coef, link, st);
-    } else {
-      b.first_item = first;
-      if (dims == 3)
-        launch_fused_batch<F32, 3>(b, total, coef, link, st);
-      else
-        launch_fused_batch<F32, 2>(b, total, coef, link, st);
+  long i = 0;
+  for (int m = kBatchModes - 1; m >= 0; --m) {
+    for (long j = 0; j < p.count[m]; ++j, ++i) {
+      b.sims = d_args + (2 * m + (i & 1)) * n;
+      b.first_item = first + m * (n + 1);
+      launch_fused_batch(b, dims, m + 1, p.items[m], coef, link, iso, st);
+      cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-// one group: same dims and field path, all batchable
+// one group: same dims, field path and isotropy, all batchable
 static dirac_status batch_group(dirac_sim* const* g, int n, long nsteps) {
   dirac_sim* s0 = g[0];
   cudaStream_t st = s0->stream;
-  // (2+1)D groups take two steps per pass for pairs of steps, as stepping alone
-  bool tb = s0->dims == 2 && nsteps >= 2 && std::getenv("DIRAC_NO_TEMPORAL_BLOCKING") == nullptr;
-  for (int i = 0; i < n && tb; ++i) tb = g[i]->tblock != 0;
-  const long pairs = tb ? nsteps / 2 : 0;
-  const long launches = pairs + (nsteps - 2 * pairs);
-  std::vector<int> chunks(2 * n);
+  // (2+1)D groups take several steps per pass, as stepping alone: as many as
+  // every member's grid allows
+  BatchPasses passes;
+  long left = nsteps;
+  int deepest = 0;
+  while (left > 0) {
+    int steps = kMaxSteps2d;
+    for (int i = 0; i < n; ++i) steps = std::min(steps, steps_per_pass(g[i], left));
+    const int m = steps - 1;
+    const long c = left / steps;
+    passes.count[m] += c;
+    left -= c * steps;
+    deepest = std::max(deepest, m);
+  }
+  const long launches = passes.launches();
+  std::vector<int> chunks(kBatchModes * n, 0);
   for (int i = 0; i < n; ++i) {
     dirac_sim* s = g[i];
-    chunks[2 * i] = s->chunk1 > 0 ? s->chunk1 : fused_chunk(s->dims, s->N);
-    chunks[2 * i + 1] = s->chunk2 > 0 ? s->chunk2 : (tb ? fused_chunk_tb2(s->N) : 0);
+    for (int m = 0; m < kBatchModes; ++m) {
+      if (!passes.count[m]) continue;
+      const int planned = m ? s->chunk2 : s->chunk1;
+      chunks[kBatchModes * i + m] = planned > 0 ? planned : fused_chunk(s->dims, s->N, m + 1);
+    }
   }
   const bool use_graph = launches <= kBatchGraphMaxLaunches && std::getenv("DIRAC_NO_GRAPHS") == nullptr;
 
@@ -1193,7 +1223,7 @@ static dirac_status batch_group(dirac_sim* const* g, int n, long nsteps) {
   if (use_graph) {  // a recorded loop of this very call?
     std::lock_guard<std::mutex> lock(g_bg_mu);
     for (BatchGraph& e : g_bgraphs) {
-      if (e.nsteps != nsteps || e.tb != (int)tb || e.sims.size() != (size_t)n || e.chunks != chunks) continue;
+      if (e.nsteps != nsteps || e.deepest != deepest || e.sims.size() != (size_t)n || e.chunks != chunks) continue;
       bool same = true;
       for (int i = 0; i < n && same; ++i) same = e.sims[i] == g[i] && e.states[i] == g[i]->state;
       if (!same) continue;
@@ -1203,18 +1233,16 @@ static dirac_status batch_group(dirac_sim* const* g, int n, long nsteps) {
     }
   }
 
-  // argument tables [mode][buffer parity][sim] (mode 0 one step per pass, 1
-  // two steps) and item prefix sums [mode][n + 1]
-  const size_t args_bytes = (size_t)4 * n * sizeof(FusedArgs<F32>);
-  const size_t first_bytes = (size_t)2 * (n + 1) * sizeof(long long);
-  std::vector<FusedArgs<F32>> h_args(4 * (size_t)n);
-  std::vector<long long> h_first(2 * (size_t)(n + 1), 0);
+  const size_t args_bytes = (size_t)2 * kBatchModes * n * sizeof(FusedArgs<F32>);
+  const size_t first_bytes = (size_t)kBatchModes * (n + 1) * sizeof(long long);
+  std::vector<FusedArgs<F32>> h_args(2 * kBatchModes * (size_t)n);
+  std::vector<long long> h_first(kBatchModes * (size_t)(n + 1), 0);
   for (int i = 0; i < n; ++i) {
     dirac_sim* s = g[i];
-    for (int mode = 0; mode < 2; ++mode) {
+    for (int m = 0; m < kBatchModes; ++m) {
       for (int p = 0; p < 2; ++p) {
         FusedArgs<F32> a = fused_args<F32>(s, sim_time(s));
-        a.chunk = chunks[2 * i + mode];
+        a.chunk = chunks[kBatchModes * i + m];
         if (p == 1) {
           for (int k = 0; k < 4; ++k) {  // the other buffer is the input after an odd launch
             float4* tmp = a.out[k];
@@ -1222,13 +1250,14 @@ static dirac_status batch_group(dirac_sim* const* g, int n, long nsteps) {
             a.in[k] = tmp;
           }
         }
-        h_args[(mode * 2 + p) * (size_t)n + i] = a;
+        h_args[(m * 2 + p) * (size_t)n + i] = a;
       }
+      if (passes.count[m])
+        h_first[m * (size_t)(n + 1) + i + 1] = h_first[m * (size_t)(n + 1) + i] +
+                                               fused_items(s->dims, s->N, m + 1, chunks[kBatchModes * i + m]);
     }
-    h_first[i + 1] = h_first[i] + fused_items(s->dims, s->N, chunks[2 * i]);
-    h_first[n + 1 + i + 1] = h_first[n + 1 + i] + (tb ? fused_items_tb2(s->N, chunks[2 * i + 1]) : 0);
   }
-  const long long total = h_first[n], total2 = h_first[2 * (size_t)n + 1];
+  for (int m = 0; m < kBatchModes; ++m) passes.items[m] = h_first[m * (size_t)(n + 1) + n];
   void* d = nullptr;
   cudaError_t e = cudaMalloc(&d, args_bytes + first_bytes);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d, h_args.data(), args_bytes, cudaMemcpyHostToDevice, st);
@@ -1250,8 +1279,7 @@ static dirac_status batch_group(dirac_sim* const* g, int n, long nsteps) {
     bool ok = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess;
     if (ok) {
       ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeRelaxed) == cudaSuccess;
-      cudaError_t le = ok ? enqueue_batch(d_args, d_first, n, pairs, launches, total, total2, s0->dims,
-                                          s0->coef_mode, s0->link_mode, cap)
+      cudaError_t le = ok ? enqueue_batch(d_args, d_first, n, passes, s0->dims, s0->coef_mode, s0->link_mode, s0->iso, cap)
                           : cudaSuccess;
       if (ok) ok = cudaStreamEndCapture(cap, &graph) == cudaSuccess && le == cudaSuccess && graph;
       if (ok) ok = cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
@@ -1271,7 +1299,7 @@ static dirac_status batch_group(dirac_sim* const* g, int n, long nsteps) {
       for (int i = 0; i < n; ++i) ent.states.push_back(g[i]->state);
       ent.chunks = chunks;
       ent.nsteps = nsteps;
-      ent.tb = (int)tb;
+      ent.deepest = deepest;
       ent.tables = d;
       ent.exec = exec;
       ent.stream = st;
@@ -1289,8 +1317,7 @@ static dirac_status batch_group(dirac_sim* const* g, int n, long nsteps) {
       return finish();
     }
   }
-  e = enqueue_batch(d_args, d_first, n, pairs, launches, total, total2, s0->dims, s0->coef_mode,
-                    s0->link_mode, st);
+  e = enqueue_batch(d_args, d_first, n, passes, s0->dims, s0->coef_mode, s0->link_mode, s0->iso, st);
   cudaStreamSynchronize(st);
   cudaFree(d);
   if (e != cudaSuccess) return cuda_fail(s0, e, "batched fused launch");
@@ -1335,7 +1362,7 @@ static dirac_status batch_step_impl(dirac_sim* const* sims, int nsims, long nste
     for (int j = i; j < nsims; ++j) {
       dirac_sim* t = sims[j];
       if (!done[j] && batchable(t) && t->dims == s->dims && t->coef_mode == s->coef_mode &&
-          t->link_mode == s->link_mode) {
+          t->link_mode == s->link_mode && t->iso == s->iso) {
         grp.push_back(t);
         done[j] = 1;
       }
@@ -1363,7 +1390,7 @@ static dirac_status observe_launch(dirac_sim* s, int dens_axis, int dens_X, doub
   a.f = field_desc(s);
   a.t_links = sim_time(s) - s->dt / 2.0;
   if (s->link_mode == LINK_PLANE) {
-    launch_link_table<P>(s->wave, s->ltab_n, a.f, s->dims, s->ltab_axis, s->f.Apw_pol, a.t_links, a.t_links,
+    launch_link_table<P>(s->wave, s->ltab_n, a.f, s->dims, s->ltab_axis, s->f.Apw_pol, &a.t_links, &a.t_links, 1,
                          s->stream);
     s->launches += 1;
     CK(s, cudaGetLastError());
@@ -1476,16 +1503,16 @@ extern "C" dirac_status dirac_set_plan(dirac_sim* s, const dirac_plan* plan) {
 
 // Time `reps` launches of one candidate (after one untimed launch) on the
 // current state, out of place into the spare buffer; milliseconds per launch.
-static dirac_status time_candidate(dirac_sim* s, int two_step, int chunk, int reps, cudaEvent_t e0,
+static dirac_status time_candidate(dirac_sim* s, int steps, int chunk, int reps, cudaEvent_t e0,
                                    cudaEvent_t e1, float* ms) {
   FusedArgs<F32> a = fused_args<F32>(s, sim_time(s));
   a.chunk = chunk;
   for (int r = 0; r <= reps; ++r) {
     if (r == 1) CK(s, cudaEventRecord(e0, s->stream));
-    const int blocks = two_step ? launch_fused2d_tb2(a, s->stream)
-                                : (s->dims == 3 ? launch_fused<F32, 3>(a, s->stream)
-                                                : launch_fused<F32, 2>(a, s->stream));
-    if (!blocks) return fail(s, DIRAC_ERR_UNSUPPORTED, "no two-step kernel for these fields");
+    const int blocks = steps > 1 ? launch_fused2d_two(a, s->stream)
+                                 : (s->dims == 3 ? launch_fused<F32, 3>(a, s->stream)
+                                                 : launch_fused<F32, 2>(a, s->stream));
+    if (!blocks) return fail(s, DIRAC_ERR_UNSUPPORTED, "no kernel of several steps for these fields");
     s->launches += 1;
     CK(s, cudaGetLastError());
   }
@@ -1505,16 +1532,14 @@ extern "C" dirac_status dirac_autotune(dirac_sim* s, dirac_plan* out) {
   }
   constexpr int kCandidates = 6;
   int c1[kCandidates], c2[kCandidates];
-  const int n1 = fused_candidates(s->dims, s->N, 0, c1, kCandidates);
-  const bool tb_ok = s->dims == 2 && s->zlo == 0 && s->nzu == s->Nzg && !time_dependent_fields(s) &&
-                     (s->coef_mode == COEF_UNIFORM || s->coef_mode == COEF_STEP ||
-                      s->coef_mode == COEF_TABLE || s->coef_mode == COEF_SOFTCORE ||
-                      s->coef_mode == COEF_SOFTCORR) &&
-                     (s->link_mode == LINK_NONE || s->link_mode == LINK_CONST) &&
-                     !((s->coef_mode == COEF_TABLE || s->coef_mode == COEF_SOFTCORE ||
-                        s->coef_mode == COEF_SOFTCORR) && s->link_mode == LINK_CONST);
-  const int n2 = tb_ok ? fused_candidates(2, s->N, 1, c2, kCandidates) : 0;
-  link_table<F32>(s, sim_time(s), s->stream);  // plane-wave links of the current step, if any
+  const int n1 = fused_candidates(s->dims, s->N, 1, c1, kCandidates);
+  // the deepest pass these fields and this grid allow, whatever the current plan says
+  const int tblock = s->tblock;
+  if (s->dims == 2) s->tblock = 1;
+  const int deep = steps_per_pass(s, kMaxSteps2d);
+  s->tblock = tblock;
+  const int n2 = deep > 1 ? fused_candidates(2, s->N, deep, c2, kCandidates) : 0;
+  link_table<F32>(s, deep, s->stream);  // plane-wave links of the current step(s), if any
   cudaEvent_t e0, e1;
   CK(s, cudaEventCreate(&e0));
   cudaError_t ce = cudaEventCreate(&e1);
@@ -1524,7 +1549,7 @@ extern "C" dirac_status dirac_autotune(dirac_sim* s, dirac_plan* out) {
   }
   // repetitions: about a millisecond of launches per candidate and sweep
   float t0 = 0.0f;
-  dirac_status st = time_candidate(s, 0, c1[0], 1, e0, e1, &t0);
+  dirac_status st = time_candidate(s, 1, c1[0], 1, e0, e1, &t0);
   int reps = 2;
   if (st == DIRAC_OK && t0 > 0.0f) reps = (int)std::ceil(1.0f / t0);
   reps = reps < 2 ? 2 : (reps > 50 ? 50 : reps);
@@ -1533,13 +1558,13 @@ extern "C" dirac_status dirac_autotune(dirac_sim* s, dirac_plan* out) {
   for (int sweep = 0; sweep < 2 && st == DIRAC_OK; ++sweep) {
     for (int i = 0; i < n1 && st == DIRAC_OK; ++i) {
       float ms = 0.0f;
-      st = time_candidate(s, 0, c1[i], reps, e0, e1, &ms);
+      st = time_candidate(s, 1, c1[i], reps, e0, e1, &ms);
       if (ms < best1[i]) best1[i] = ms;
     }
     for (int i = 0; i < n2 && st == DIRAC_OK; ++i) {
       float ms = 0.0f;
-      st = time_candidate(s, 1, c2[i], reps, e0, e1, &ms);
-      if (ms / 2.0f < best2[i]) best2[i] = ms / 2.0f;  // two steps per launch
+      st = time_candidate(s, deep, c2[i], reps, e0, e1, &ms);
+      if (ms / (float)deep < best2[i]) best2[i] = ms / (float)deep;  // several steps per launch
     }
   }
   cudaEventDestroy(e0);
@@ -1557,7 +1582,7 @@ extern "C" dirac_status dirac_autotune(dirac_sim* s, dirac_plan* out) {
     p.two_step = best2[i2] < best1[i1] ? 1 : 0;
     if (p.two_step) p.us_per_step = 1e3 * best2[i2];
   } else if (s->dims == 2) {
-    p.two_step = s->tblock;  // fields that never take two-step passes: keep the flag as it was
+    p.two_step = s->tblock;  // fields that never take passes of several steps: keep the flag as it was
   }
   drop_graphs(s);
   apply_plan(s, p);

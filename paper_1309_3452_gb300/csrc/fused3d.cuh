@@ -161,7 +161,7 @@ __host__ __device__ __forceinline__ long long items3d(const int (&N)[3], int lev
 // y neighbour of a cell inside the pair comes from the other cell's registers;
 // the pair's outer y neighbours and all x neighbours come from shared memory.
 // `a` may live in the constant bank (kernel parameter) or in shared memory.
-template <class P, int COEF, int LINK, bool kE, int kPairs>
+template <class P, int COEF, int LINK, bool kE, int kPairs, bool kIso>
 __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long item, const Thread3d& th,
                                              unsigned char* smem_raw, double* e_acc) {
   using T = Tile3<kPairs>;
@@ -293,7 +293,7 @@ __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long it
     dn[2] = zd;
     SoftB2 b;
     if constexpr (kSoft) b = pair_b(h, cell, xy, zq, H0, H1, rec, 2 * comp);
-    return quad_update<3, COEF, LINK, true>(h, a.f, iso, a.ry, a.rz, comp, F, up, dn, H0, H1, site, site, a.pstride, S,
+    return quad_update<3, COEF, LINK, true, kIso>(h, a.f, iso, a.ry, a.rz, comp, F, up, dn, H0, H1, site, site, a.pstride, S,
                                             kSoft ? &b : nullptr, lk, a.N);
   };
 
@@ -436,7 +436,7 @@ __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long it
 
 // kE: the launch also accumulates the conserved functional of the new state (a
 // kernel of its own, so that the others carry neither its terms nor its tests)
-template <class P, int COEF, int LINK, bool kE, int kPairs>
+template <class P, int COEF, int LINK, bool kE, int kPairs, bool kIso>
 __global__ void __launch_bounds__(Tile3<kPairs>::threads, 1) fused3d_kernel(const FusedArgs<P> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int kThreads3d = Tile3<kPairs>::threads;
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(Tile3<kPairs>::threads, 1) fused3d_kernel(cons
   double* acc = e_acc[kE ? threadIdx.x : 0];
   if (kE) acc[0] = acc[1] = 0.0;
   for (long long item = blockIdx.x; item < items; item += a.workers)
-    fused3d_item<P, COEF, LINK, kE, kPairs>(a, item, th, smem_raw, acc);
+    fused3d_item<P, COEF, LINK, kE, kPairs, kIso>(a, item, th, smem_raw, acc);
   if (kE) block_store_e(acc[0], acc[1], a.e_partials);
 }
 
@@ -459,7 +459,7 @@ constexpr int kBatchPairs = 14;
 // Several simulations in one persistent launch: global items are the
 // simulations' items back to back; each block copies the arguments of the
 // simulation its current item belongs to into shared memory.
-template <class P, int COEF, int LINK>
+template <class P, int COEF, int LINK, bool kIso>
 __global__ void __launch_bounds__(Tile3<kBatchPairs>::threads, 1) fused3d_batch_kernel(const BatchArgs<P> b) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ FusedArgs<P> sa;
@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(Tile3<kBatchPairs>::threads, 1) fused3d_batch_
       cur = s;
     }
     // (batched launches never accumulate the functional: e_partials is null)
-    fused3d_item<P, COEF, LINK, false, kBatchPairs>(sa, g - b.first_item[s], th, smem_raw, nullptr);
+    fused3d_item<P, COEF, LINK, false, kBatchPairs, kIso>(sa, g - b.first_item[s], th, smem_raw, nullptr);
   }
 }
 
@@ -502,16 +502,16 @@ bool taller_tile(const int N[3]) {
   const long long r15 = (N[1] + Tile3<15>::CY - 1) / Tile3<15>::CY * Tile3<15>::TH;
   return COEF == COEF_SOFTCORE ? 95 * r15 < 100 * r14 : r15 < r14;
 }
-// the field paths built with both tiles (the others, and the launches that
-// accumulate the functional, run with 14 pairs)
+// the field paths built with both tiles (the others, the launches that
+// accumulate the functional and anisotropic grids run with 14 pairs)
 template <int COEF, int LINK>
 constexpr bool both_tiles() {
   return COEF != kAnyMode && COEF != COEF_SOFTCORR && LINK != LINK_TABLE;
 }
 
-template <int COEF, int LINK, bool kE, int kPairs>
+template <int COEF, int LINK, bool kE, int kPairs, bool kIso>
 int launch3d_tile(FusedArgs<F32> a, cudaStream_t s) {
-  constexpr auto k = fused3d_kernel<F32, COEF, LINK, kE, kPairs>;
+  constexpr auto k = fused3d_kernel<F32, COEF, LINK, kE, kPairs, kIso>;
   const int resident = workers3d<k, kPairs>();
   if (a.chunk <= 0 || a.chunk > a.nzu) a.chunk = plan_chunk(ChunkShape{tiles3d<kPairs>(a.N), a.nzu, resident, 4, 0.5});
   const long long items = items3d<kPairs>(a.N, a.nzu, a.chunk);
@@ -524,15 +524,20 @@ int launch3d_tile(FusedArgs<F32> a, cudaStream_t s) {
 
 template <int COEF, int LINK>
 int launch3d(FusedArgs<F32> a, cudaStream_t s) {
-  if (a.e_partials) return launch3d_tile<COEF, LINK, true, 14>(a, s);
+  if constexpr (COEF != kAnyMode) {  // (the run-time path tests iso itself)
+    if (!a.iso)
+      return a.e_partials ? launch3d_tile<COEF, LINK, true, 14, false>(a, s)
+                          : launch3d_tile<COEF, LINK, false, 14, false>(a, s);
+  }
+  if (a.e_partials) return launch3d_tile<COEF, LINK, true, 14, true>(a, s);
   if constexpr (both_tiles<COEF, LINK>())
-    if (taller_tile<COEF>(a.N)) return launch3d_tile<COEF, LINK, false, 15>(a, s);
-  return launch3d_tile<COEF, LINK, false, 14>(a, s);
+    if (taller_tile<COEF>(a.N)) return launch3d_tile<COEF, LINK, false, 15, true>(a, s);
+  return launch3d_tile<COEF, LINK, false, 14, true>(a, s);
 }
 
-template <int COEF, int LINK>
+template <int COEF, int LINK, bool kIso>
 void launch3d_batch(BatchArgs<F32> b, long long total, cudaStream_t s) {
-  constexpr auto k = fused3d_batch_kernel<F32, COEF, LINK>;
+  constexpr auto k = fused3d_batch_kernel<F32, COEF, LINK, kIso>;
   const int resident = workers3d<k, kBatchPairs>();
   b.workers = (int)(total < resident ? total : resident);
   k<<<(unsigned)b.workers, Tile3<kBatchPairs>::threads, Tile3<kBatchPairs>::smem, s>>>(b);

@@ -7,14 +7,9 @@ namespace fused {
 ChunkShape shape3d(const int N[3]) {
   const int n[3] = {N[0], N[1], N[2]};
   return {tiles3d<kBatchPairs>(n), N[2],
-          workers3d<fused3d_kernel<F32, COEF_UNIFORM, LINK_NONE, false, kBatchPairs>, kBatchPairs>(), 4, 0.5};
+          workers3d<fused3d_kernel<F32, COEF_UNIFORM, LINK_NONE, false, kBatchPairs, true>, kBatchPairs>(), 4, 0.5};
 }
 
-#define BATCH_3D(COEF, LINK) template void launch3d_batch<COEF, LINK>(BatchArgs<F32>, long long, cudaStream_t);
-BATCH_3D(COEF_UNIFORM, LINK_NONE)
-BATCH_3D(COEF_STEP, LINK_NONE)
-BATCH_3D(COEF_UNIFORM, LINK_CONST)
-BATCH_3D(COEF_STEP, LINK_CONST)
 #define STEP_3D(COEF, LINK) template int launch3d<COEF, LINK>(FusedArgs<F32>, cudaStream_t);
 STEP_3D(COEF_UNIFORM, LINK_NONE)
 STEP_3D(COEF_STEP, LINK_NONE)

@@ -98,8 +98,7 @@ struct ChunkShape {
   double restart;
 };
 ChunkShape shape3d(const int N[3]);
-ChunkShape shape2d(const int N[3]);
-ChunkShape shape2d_tb2(const int N[3]);
+ChunkShape shape2d(const int N[3], int steps);  // steps per pass
 // chunk length (levels per item) by that rule
 int plan_chunk(const ChunkShape& g);
 

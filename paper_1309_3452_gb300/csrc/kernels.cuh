@@ -35,6 +35,7 @@ struct FusedArgs {
   int iso;
   typename P::Ratio ry, rz;
   HalfFields<P> hu, hl;     // upper / lower half-step fields
+  int lstep;                // LINK_PLANE: table entries from one time step of a pass to the next
   FieldDesc f;
   // non-null: accumulate the conserved functional of the new state (per block
   // [sum |psi|^2, Re sum_lower conj(G) S'_G]; E = first + r_x second)
@@ -45,24 +46,24 @@ struct FusedArgs {
   // A whole grid: zlo = 0, nzu = Nzg = N[axis], zorg = 0 (periodic wrap of
   // the stored levels); a slab of a decomposed grid: its own levels between
   // one halo level on either side (zlo = 1, nzu = N[axis] - 2), zorg = its
-  // first global level - 1.  (The two-step (2+1)D kernel and the batched
-  // kernels take whole grids only.)
+  // first global level - 1.  (Passes of several steps and the batched kernels
+  // take whole grids only.)
   int zlo, nzu, zorg, Nzg;
 };
 constexpr int kFusedEMaxBlocks = 4096;  // capacity of the per-block E partials
 // (2+1)D fused kernel geometry
-constexpr int kFused2dWarps = 8;   // independent x strips per block
-constexpr int kCore = 30;          // interior lanes of a 32-lane strip
+constexpr int kFused2dWarps = 4;   // independent x strips per block (few, so that small grids spread over the SMs)
+constexpr int kMaxSteps2d = 2;     // most time steps per pass
 
 // returns the number of blocks launched
 template <class P, int DIMS>
 int launch_fused(const FusedArgs<P>& a, cudaStream_t s);
 
-// Two time steps per pass of the (2+1)D fused kernel (fields without time
-// dependence: uniform / Klein-step / soft-core coefficients, no or constant
-// links).  Returns the number of blocks launched, or 0, launching nothing,
-// for other field paths.
-int launch_fused2d_tb2(const FusedArgs<F32>& a, cudaStream_t s);
+// Two time steps per pass of the (2+1)D fused kernel, for every field path but
+// the per-site ones; plane waves take one link table per step (lstep).  Grids
+// of at least four rows.  Returns the number of blocks
+// launched, or 0, launching nothing, for the per-site field paths.
+int launch_fused2d_two(const FusedArgs<F32>& a, cudaStream_t s);
 
 // Several simulations (same dims and time-independent field modes) in one
 // persistent launch of the fused kernels.
@@ -74,22 +75,15 @@ struct BatchArgs {
   int workers;                   // set by the launcher
 };
 // levels per work item and number of items the fused kernels use for a grid
-// (a FusedArgs chunk of 0 makes the launchers take fused_chunk's rule)
-int fused_chunk(int dims, const int N[3]);
-// chunk lengths worth timing, best first by the planner's model, for the
-// one-step kernels or (two_step, (2+1)D) the two-step kernel; returns the count
-int fused_candidates(int dims, const int N[3], int two_step, int* out, int max);
-long long fused_items(int dims, const int N[3], int chunk);
-template <class P, int DIMS>
-void launch_fused_batch(const BatchArgs<P>& b, long long total_items, int coef_mode, int link_mode,
-                        cudaStream_t s);
-// (2+1)D two steps per pass: rows per item by the rule, items of a grid, and
-// the batched launch (uniform / Klein-step coefficients, no / constant links)
-int fused_chunk_tb2(const int N[3]);
-long long fused_items_tb2(const int N[3], int chunk);
-void launch_fused2d_tb2_batch(const BatchArgs<F32>& b, long long total_items, int coef_mode, int link_mode,
-                              cudaStream_t s);
-
+// (a FusedArgs chunk of 0 makes the launchers take fused_chunk's rule), with
+// `steps` time steps per pass (1; (2+1)D: 1 or 2)
+int fused_chunk(int dims, const int N[3], int steps);
+// chunk lengths worth timing, best first by the planner's model; returns the count
+int fused_candidates(int dims, const int N[3], int steps, int* out, int max);
+long long fused_items(int dims, const int N[3], int steps, int chunk);
+// one launch: uniform / Klein-step coefficients, no / constant links, all members isotropic or none
+void launch_fused_batch(const BatchArgs<F32>& b, int dims, int steps, long long total_items, int coef_mode,
+                        int link_mode, bool iso, cudaStream_t s);
 // Observables of the stored state: per-block FP64 partial sums of
 // [sum|psi|^2, Bx, By, Bz, sum_{beyond} |psi|^2] with
 // B_a = Re sum_lower conj(G) s_a d_a(G)  (E = naive + r_x Bx + r_y By + r_z Bz).
@@ -128,9 +122,10 @@ void launch_finish_sums2(const double* partials, int nblocks, double* out, cudaS
 // table of plane-wave link factors exp(-i phi) for both half-steps of one time
 // step: tab[half * n + H], H = half-lattice coordinate along `axis`, n = 2 N_axis;
 // elements of PlaneLinkOf<P>::type
+// (steps tables of consecutive time steps one after another, t_up and t_lo given per step)
 template <class P>
-void launch_link_table(void* tab, int n, const FieldDesc& f, int dims, int axis, int pol, double t_up,
-                       double t_lo, cudaStream_t s);
+void launch_link_table(void* tab, int n, const FieldDesc& f, int dims, int axis, int pol, const double* t_up,
+                       const double* t_lo, int steps, cudaStream_t s);
 
 // coefficient table of a time-independent potential (COEF_TABLE): every
 // plane of the state layout (pstride), b = 1/(1 + i dt (beta m + V)/2) as

@@ -240,9 +240,9 @@ __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
           for (int ax = 0; ax < DIMS; ++ax) {  // (an index known at compile time)
             if (ax != a.f.Apw_pol) continue;
             if constexpr (sizeof(R) == 4) {
-              const PlaneLink32* f = static_cast<const PlaneLink32*>(a.wave) + h;
-              sum[1 + ax].add_product(__ldg(&f->ch.x), __ldg(&f->cl.x), pt);
-              sum[1 + ax].add_product(__ldg(&f->sp.x), __ldg(&f->lp.x), qt);
+              const float4 f = __ldg(&(static_cast<const PlaneLink32*>(a.wave) + h)->v);
+              sum[1 + ax].add_product(f.x, f.y, pt);
+              sum[1 + ax].add_product(f.z, f.w, qt);
             } else {
               const double2 f = __ldg(static_cast<const double2*>(a.wave) + h);  // (cos phi, -sin phi)
               sum[1 + ax].add(f.x * pt - f.y * qt);
@@ -283,6 +283,7 @@ __device__ __forceinline__ void plane_link_from(double phi, PlaneLink32* out) {
   sincos(phi, &sn, &cs);
   const float ch = __double2float_rn(cs), sh = __double2float_rn(sn);
   const float cl = __double2float_rn(cs - (double)ch), sl = __double2float_rn(sn - (double)sh);
+  out->v = make_float4(ch, cl, sh, sl);
   out->ch = make_float2(ch, ch);
   out->cl = make_float2(cl, cl);
   out->sh = make_float2(sh, -sh);
@@ -300,16 +301,19 @@ __device__ __forceinline__ void store_quad_lane(float4* rec, int lane, float4 v)
   r[6] = v.w;
 }
 
+struct LinkTimes {
+  double up[kMaxSteps2d], lo[kMaxSteps2d];
+};
 template <class P>
 __global__ void link_table_kernel(typename PlaneLinkOf<P>::type* tab, int n, const FieldDesc f, int dims,
-                                  int axis, int pol, double t_up, double t_lo) {
+                                  int axis, int pol, const LinkTimes t, int steps) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 2 * n) return;
-  const int half = i / n;
+  if (i >= 2 * n * steps) return;
+  const int step = i / (2 * n), j = i - step * 2 * n, half = j / n;
   long long HH[3] = {0, 0, 0};
-  HH[axis] = i - half * n;
+  HH[axis] = j - half * n;
   // the same phase function as the per-link FP64 path
-  plane_link_from(link_phase(f, dims, HH, pol, +1, half ? t_lo : t_up), tab + i);
+  plane_link_from(link_phase(f, dims, HH, pol, +1, half ? t.lo[step] : t.up[step]), tab + i);
 }
 
 // b = 1/(1 + i theta), theta = dt (beta m + V)/2 with V complex, of every site
@@ -611,13 +615,20 @@ template int launch_observables<F32, 2>(const ObsArgs<F32>&, int, cudaStream_t);
 template int launch_observables<F32, 3>(const ObsArgs<F32>&, int, cudaStream_t);
 
 template <class P>
-void launch_link_table(void* tab, int n, const FieldDesc& f, int dims, int axis, int pol, double t_up,
-                       double t_lo, cudaStream_t s) {
-  link_table_kernel<P><<<(2 * n + 127) / 128, 128, 0, s>>>(static_cast<typename PlaneLinkOf<P>::type*>(tab),
-                                                           n, f, dims, axis, pol, t_up, t_lo);
+void launch_link_table(void* tab, int n, const FieldDesc& f, int dims, int axis, int pol, const double* t_up,
+                       const double* t_lo, int steps, cudaStream_t s) {
+  LinkTimes t{};
+  for (int j = 0; j < steps; ++j) {
+    t.up[j] = t_up[j];
+    t.lo[j] = t_lo[j];
+  }
+  link_table_kernel<P><<<(2 * n * steps + 127) / 128, 128, 0, s>>>(
+      static_cast<typename PlaneLinkOf<P>::type*>(tab), n, f, dims, axis, pol, t, steps);
 }
-template void launch_link_table<F64>(void*, int, const FieldDesc&, int, int, int, double, double, cudaStream_t);
-template void launch_link_table<F32>(void*, int, const FieldDesc&, int, int, int, double, double, cudaStream_t);
+template void launch_link_table<F64>(void*, int, const FieldDesc&, int, int, int, const double*, const double*, int,
+                                     cudaStream_t);
+template void launch_link_table<F32>(void*, int, const FieldDesc&, int, int, int, const double*, const double*, int,
+                                     cudaStream_t);
 
 void launch_coef_table(float4* tab, const FieldDesc& f, int dims, const int N[3], long long pstride, int quads,
                        cudaStream_t s) {

@@ -82,10 +82,10 @@ __device__ __forceinline__ Quad plane_link_diff(float2 ch, float2 cl, float2 sp,
 }
 
 // combine<F32, DIMS> of both values
-template <int DIMS>
-__device__ __forceinline__ Quad combine_quad(const Quad& dx, const Quad& dy, const Quad& dz, int p, bool iso,
+template <int DIMS, bool kIso>
+__device__ __forceinline__ Quad combine_quad(const Quad& dx, const Quad& dy, const Quad& dz, int p,
                                              const F32::Ratio& ry, const F32::Ratio& rz) {
-  if (!iso) {
+  if (!kIso) {
     const float2 tre = p ? pneg(dy.im) : dy.im, tim = p ? dy.re : pneg(dy.re);
     Quad s{padd(dx.re, ratio_mul(ry, tre)), padd(dx.im, ratio_mul(ry, tim))};
     if (DIMS == 3) {
@@ -115,6 +115,36 @@ __device__ __forceinline__ Quad apply_quad(const F32::Coef& c, const Quad& F, co
   re = pfma(f2(-c.a_hi.y), F.im, re);
   im = pfma(f2(c.a_hi.y), F.re, im);
   return Quad{pfma(f2(c.a_hi.x), F.re, re), pfma(f2(c.a_hi.x), F.im, im)};
+}
+// apply of both values with coefficients of their own, from lane_coefs' records
+__device__ __forceinline__ Quad apply_lanes(const float4* t, const Quad& F, const Quad& S) {
+  const Quad ah = quad(t[0]), gh = quad(t[32]), al = quad(t[64]), gl = quad(t[96]);
+  float2 re = pmul(gl.im, S.im), im = pmul(pneg(gl.im), S.re);
+  re = pfma(pneg(gl.re), S.re, re);
+  im = pfma(pneg(gl.re), S.im, im);
+  re = pfma(pneg(al.im), F.im, re);
+  im = pfma(al.im, F.re, im);
+  re = pfma(al.re, F.re, re);
+  im = pfma(al.re, F.im, im);
+  re = pfma(gh.im, S.im, re);
+  im = pfma(pneg(gh.im), S.re, im);
+  re = pfma(pneg(gh.re), S.re, re);
+  im = pfma(pneg(gh.re), S.im, im);
+  re = pfma(pneg(ah.im), F.im, re);
+  im = pfma(ah.im, F.re, im);
+  return Quad{pfma(ah.re, F.re, re), pfma(ah.re, F.im, im)};
+}
+// a lane's four records (alpha hi, gamma hi, alpha lo, gamma lo; 32 lanes
+// interleaved) of a half-step, value l beyond the step where beyond[l]
+__device__ __forceinline__ void lane_coefs(const HalfFields<F32>& h, bool beyond0, bool beyond1, float4* t) {
+  auto rec = [&](float2 F32::Coef::*m) {
+    const float2 i = h.c_in.*m, o = h.c_out.*m;
+    return make_float4(beyond0 ? o.x : i.x, beyond1 ? o.x : i.x, beyond0 ? o.y : i.y, beyond1 ? o.y : i.y);
+  };
+  t[0] = rec(&F32::Coef::a_hi);
+  t[32] = rec(&F32::Coef::g_hi);
+  t[64] = rec(&F32::Coef::a_lo);
+  t[96] = rec(&F32::Coef::g_lo);
 }
 // w = 2F - r_x S' of both values, small product first
 __device__ __forceinline__ Quad two_f_minus_s(float rxh, float rxl, const Quad& F, const Quad& S) {
@@ -154,14 +184,19 @@ __device__ __forceinline__ float4 lanes_of(float4 r0, float4 r1) { return make_f
 // up, dn: the neighbours at +-dx_a/2 of each lane's value; H0, H1 and site0,
 // site1: each lane's half-lattice point and cell.  bpre: the coefficients of
 // the pair where the caller forms them (COEF_SOFTCORE, COEF_SOFTCORR); lk: the
-// staged link factor of LINK_PLANE_ZX.  kOneCell: site0 == site1.
-template <int DIMS, int COEF, int LINK, bool kOneCell>
+// staged link factor of LINK_PLANE_ZX; lanes: COEF_LANES; w0, w1: the lanes'
+// factors (c_hi, c_lo, s_hi, s_lo) of LINK_PLANE.
+// kOneCell: site0 == site1.  kIso: r_x = r_y = r_z (a template parameter: a
+// test here, uniform as it is, would end the compiler's basic block at every
+// component and keep it from overlapping the chains of the others).
+template <int DIMS, int COEF, int LINK, bool kOneCell, bool kIso>
 __device__ __forceinline__ Quad quad_update(const HalfFields<F32>& h, const FieldDesc& f, bool iso,
                                             const F32::Ratio& ry, const F32::Ratio& rz, int comp, const Quad& F,
                                             const Quad (&up)[3], const Quad (&dn)[3], const int (&H0)[3],
                                             const int (&H1)[3], long long site0, long long site1, long long pstride,
                                             Quad* S_out, const SoftB2* bpre, const PlaneLink32* lk,
-                                            const int (&N)[3]) {
+                                            const int (&N)[3], const float4* lanes = nullptr,
+                                            const float4* w0 = nullptr, const float4* w1 = nullptr) {
   if constexpr (COEF == kAnyMode || LINK == kAnyMode) {
     // the per-site FP64 paths and rare combinations: one value at a time
     float2 r[2], S[2];
@@ -206,13 +241,7 @@ __device__ __forceinline__ Quad quad_update(const HalfFields<F32>& h, const Fiel
     if constexpr (LINK == LINK_PLANE_ZX)  // the factor of the values' z level, staged by the caller
       d[0] = plane_link_diff(lk->ch, lk->cl, lk->sp, lk->lp, up[0], dn[0]);
     if constexpr (LINK == LINK_PLANE) {
-      // each lane's factor from the step's table
-      const PlaneLink32* tab = static_cast<const PlaneLink32*>(h.ltab);
-      const int a = h.ltab_axis;
-      const PlaneLink32 *p0 = tab + (a == 0 ? H0[0] : (a == 1 ? H0[1] : H0[2])),
-                        *p1 = tab + (a == 0 ? H1[0] : (a == 1 ? H1[1] : H1[2]));
-      const float4 v0 = make_float4(p0->ch.x, p0->cl.x, p0->sp.x, p0->lp.x);
-      const float4 v1 = make_float4(p1->ch.x, p1->cl.x, p1->sp.x, p1->lp.x);
+      const float4 v0 = *w0, v1 = *w1;  // each lane's factor
       const float2 ch = make_float2(v0.x, v1.x), cl = make_float2(v0.y, v1.y);
       const float2 sp = make_float2(v0.z, v1.z), lp = make_float2(v0.w, v1.w);
       if (h.lpol == 0) d[0] = plane_link_diff(ch, cl, sp, lp, up[0], dn[0]);
@@ -220,10 +249,14 @@ __device__ __forceinline__ Quad quad_update(const HalfFields<F32>& h, const Fiel
       else if (DIMS == 3) d[2] = plane_link_diff(ch, cl, sp, lp, up[2], dn[2]);
     }
     if (DIMS == 2) d[2] = d[0];
-    const Quad S = combine_quad<DIMS>(d[0], d[1], d[2], sign_class<DIMS>(2 * comp), iso, ry, rz);
+    const Quad S = combine_quad<DIMS, kIso>(d[0], d[1], d[2], sign_class<DIMS>(2 * comp), ry, rz);
     if (S_out) *S_out = S;
     if constexpr (COEF == COEF_UNIFORM) {
       return apply_quad(h.c_in, F, S);
+    } else if constexpr (COEF == COEF_BEYOND) {
+      return apply_quad(h.c_out, F, S);
+    } else if constexpr (COEF == COEF_LANES) {
+      return apply_lanes(lanes, F, S);
     } else if constexpr (COEF == COEF_STEP) {
       // both values on one side of the step almost everywhere: one apply, two
       // (and a choice per lane) only in the cells the step cuts

@@ -1,23 +1,19 @@
-// Planning and dispatch of the fused time-step kernels (fused3d.cuh, fused2d.cu).
+// Planning and dispatch of the fused time-step kernels (fused3d.cuh, fused2d.cuh).
 #include "fused_common.cuh"
 
 namespace dirac {
 
 namespace fused {
 
-// the launchers, instantiated per field path in fused3d_*.cu and fused2d.cu
+// the launchers, instantiated per field path in fused3d_*.cu and fused2d_*.cu
 template <int COEF, int LINK>
 int launch3d(FusedArgs<F32> a, cudaStream_t s);
-template <int COEF, int LINK>
+template <int COEF, int LINK, bool kIso>
 void launch3d_batch(BatchArgs<F32> b, long long total, cudaStream_t s);
-template <int COEF, int LINK>
+template <int COEF, int LINK, int kT>
 int launch2d(FusedArgs<F32> a, cudaStream_t s);
-template <int COEF, int LINK>
-int launch2d_tb2(FusedArgs<F32> a, cudaStream_t s);
-template <int COEF, int LINK>
+template <int COEF, int LINK, int kT, bool kIso>
 void launch2d_batch(BatchArgs<F32> b, long long total, cudaStream_t s);
-template <int COEF, int LINK>
-void launch2d_tb2_batch(BatchArgs<F32> b, long long total, cudaStream_t s);
 // Chunk length (levels per item) for `tiles` items per level chunk, `levels`
 // levels and `workers` persistent workers: maximise the busy fraction of the
 // rounds times the useful fraction chunk/(chunk+restart) of each item, where
@@ -68,128 +64,118 @@ using namespace fused;
 
 namespace {
 
-template <int DIMS, int COEF, int LINK>
+// kT time steps per pass ((3+1)D: one)
+template <int DIMS, int kT, int COEF, int LINK>
 int launch_dims(const FusedArgs<F32>& a, cudaStream_t s) {
   if constexpr (DIMS == 3) {
     // (3+1)D plane waves are dispatched before reaching here (LINK_PLANE_ZX)
     if constexpr (LINK == LINK_PLANE) return launch3d<kAnyMode, kAnyMode>(a, s);
     else return launch3d<COEF, LINK>(a, s);
+  } else if constexpr (COEF == kAnyMode && kT > 1) {
+    return 0;  // the per-site paths take one step per pass
   } else {
-    return launch2d<COEF, LINK>(a, s);
+    if constexpr (COEF == COEF_STEP)
+      if (a.hu.step_axis == 0) return launch2d<COEF_STEP_X, LINK, kT>(a, s);
+    return launch2d<COEF, LINK, kT>(a, s);
   }
 }
 
-template <int DIMS>
+template <int DIMS, int kT>
 int dispatch(const FusedArgs<F32>& a, cudaStream_t s) {
   const int c = a.hu.coef_mode, l = a.hu.link_mode;
-  if (c == COEF_GENERAL || l == LINK_GENERAL) return launch_dims<DIMS, kAnyMode, kAnyMode>(a, s);
+#define RUN(COEF, LINK) return launch_dims<DIMS, kT, COEF, LINK>(a, s)
+  if (c == COEF_GENERAL || l == LINK_GENERAL) RUN(kAnyMode, kAnyMode);
   // the fused (3+1)D kernel stages plane-wave link factors per z level: a wave
   // along z polarised along x runs as LINK_PLANE_ZX, other plane waves take
   // the general path there
-  if (DIMS == 3 && l == LINK_PLANE) {
-    if (a.hu.ltab_axis != 2 || a.hu.lpol != 0) return launch3d<kAnyMode, kAnyMode>(a, s);
-    if (c == COEF_UNIFORM) return launch3d<COEF_UNIFORM, LINK_PLANE_ZX>(a, s);
-    if (c == COEF_STEP) return launch3d<COEF_STEP, LINK_PLANE_ZX>(a, s);
-    if (c == COEF_TABLE) return launch3d<COEF_TABLE, LINK_PLANE_ZX>(a, s);
-    if (c == COEF_SOFTCORE) return launch3d<COEF_SOFTCORE, LINK_PLANE_ZX>(a, s);
-    if (c == COEF_SOFTCORR) return launch3d<COEF_SOFTCORR, LINK_PLANE_ZX>(a, s);
-    return launch3d<kAnyMode, kAnyMode>(a, s);
+  if constexpr (DIMS == 3) {
+    if (l == LINK_PLANE) {
+      if (a.hu.ltab_axis != 2 || a.hu.lpol != 0) RUN(kAnyMode, kAnyMode);
+      if (c == COEF_UNIFORM) RUN(COEF_UNIFORM, LINK_PLANE_ZX);
+      if (c == COEF_STEP) RUN(COEF_STEP, LINK_PLANE_ZX);
+      if (c == COEF_TABLE) RUN(COEF_TABLE, LINK_PLANE_ZX);
+      if (c == COEF_SOFTCORE) RUN(COEF_SOFTCORE, LINK_PLANE_ZX);
+      if (c == COEF_SOFTCORR) RUN(COEF_SOFTCORR, LINK_PLANE_ZX);
+      RUN(kAnyMode, kAnyMode);
+    }
   }
   if (c == COEF_SOFTCORE) {
-    if (l == LINK_NONE) return launch_dims<DIMS, COEF_SOFTCORE, LINK_NONE>(a, s);
-    if (l == LINK_PLANE) return launch_dims<DIMS, COEF_SOFTCORE, LINK_PLANE>(a, s);
-    return launch_dims<DIMS, kAnyMode, kAnyMode>(a, s);
+    if (l == LINK_NONE) RUN(COEF_SOFTCORE, LINK_NONE);
+    if (l == LINK_PLANE) RUN(COEF_SOFTCORE, LINK_PLANE);
+    RUN(kAnyMode, kAnyMode);
   }
   if (c == COEF_SOFTCORR) {
-    if (l == LINK_NONE) return launch_dims<DIMS, COEF_SOFTCORR, LINK_NONE>(a, s);
-    if (l == LINK_PLANE) return launch_dims<DIMS, COEF_SOFTCORR, LINK_PLANE>(a, s);
-    return launch_dims<DIMS, kAnyMode, kAnyMode>(a, s);
+    if (l == LINK_NONE) RUN(COEF_SOFTCORR, LINK_NONE);
+    if (l == LINK_PLANE) RUN(COEF_SOFTCORR, LINK_PLANE);
+    RUN(kAnyMode, kAnyMode);
   }
   if (l == LINK_TABLE) {
-    if (c == COEF_UNIFORM) return launch_dims<DIMS, COEF_UNIFORM, LINK_TABLE>(a, s);
-    if (c == COEF_STEP) return launch_dims<DIMS, COEF_STEP, LINK_TABLE>(a, s);
-    return launch_dims<DIMS, COEF_TABLE, LINK_TABLE>(a, s);
+    if (c == COEF_UNIFORM) RUN(COEF_UNIFORM, LINK_TABLE);
+    if (c == COEF_STEP) RUN(COEF_STEP, LINK_TABLE);
+    RUN(COEF_TABLE, LINK_TABLE);
   }
-  if (c == COEF_TABLE && l == LINK_NONE) return launch_dims<DIMS, COEF_TABLE, LINK_NONE>(a, s);
-  if (c == COEF_TABLE && l == LINK_PLANE) return launch_dims<DIMS, COEF_TABLE, LINK_PLANE>(a, s);
-  if (c == COEF_TABLE) return launch_dims<DIMS, kAnyMode, kAnyMode>(a, s);
-  if (c == COEF_UNIFORM && l == LINK_PLANE) return launch_dims<DIMS, COEF_UNIFORM, LINK_PLANE>(a, s);
-  if (c == COEF_STEP && l == LINK_PLANE) return launch_dims<DIMS, COEF_STEP, LINK_PLANE>(a, s);
-  if (c == COEF_UNIFORM && l == LINK_NONE) return launch_dims<DIMS, COEF_UNIFORM, LINK_NONE>(a, s);
-  if (c == COEF_STEP && l == LINK_NONE) return launch_dims<DIMS, COEF_STEP, LINK_NONE>(a, s);
-  if (c == COEF_UNIFORM && l == LINK_CONST) return launch_dims<DIMS, COEF_UNIFORM, LINK_CONST>(a, s);
-  return launch_dims<DIMS, COEF_STEP, LINK_CONST>(a, s);
+  if (c == COEF_TABLE && l == LINK_NONE) RUN(COEF_TABLE, LINK_NONE);
+  if (c == COEF_TABLE && l == LINK_PLANE) RUN(COEF_TABLE, LINK_PLANE);
+  if (c == COEF_TABLE) RUN(kAnyMode, kAnyMode);
+  if (c == COEF_UNIFORM && l == LINK_PLANE) RUN(COEF_UNIFORM, LINK_PLANE);
+  if (c == COEF_STEP && l == LINK_PLANE) RUN(COEF_STEP, LINK_PLANE);
+  if (c == COEF_UNIFORM && l == LINK_NONE) RUN(COEF_UNIFORM, LINK_NONE);
+  if (c == COEF_STEP && l == LINK_NONE) RUN(COEF_STEP, LINK_NONE);
+  if (c == COEF_UNIFORM && l == LINK_CONST) RUN(COEF_UNIFORM, LINK_CONST);
+  RUN(COEF_STEP, LINK_CONST);
+#undef RUN
 }
 
-template <int DIMS, int COEF, int LINK>
-void batch_dims(const BatchArgs<F32>& b, long long total, cudaStream_t s) {
-  if (DIMS == 3) launch3d_batch<COEF, LINK>(b, total, s);
-  else launch2d_batch<COEF, LINK>(b, total, s);
+template <int DIMS, int kT, int COEF, int LINK>
+void batch_dims(const BatchArgs<F32>& b, long long total, bool iso, cudaStream_t s) {
+  if constexpr (DIMS == 3) {
+    if (iso) launch3d_batch<COEF, LINK, true>(b, total, s);
+    else launch3d_batch<COEF, LINK, false>(b, total, s);
+  } else {
+    if (iso) launch2d_batch<COEF, LINK, kT, true>(b, total, s);
+    else launch2d_batch<COEF, LINK, kT, false>(b, total, s);
+  }
 }
+template <int DIMS, int kT>
+void dispatch_batch(const BatchArgs<F32>& b, long long total, int coef, int link, bool iso, cudaStream_t s) {
+  if (coef == COEF_UNIFORM && link == LINK_NONE) batch_dims<DIMS, kT, COEF_UNIFORM, LINK_NONE>(b, total, iso, s);
+  else if (coef == COEF_STEP && link == LINK_NONE) batch_dims<DIMS, kT, COEF_STEP, LINK_NONE>(b, total, iso, s);
+  else if (coef == COEF_UNIFORM && link == LINK_CONST) batch_dims<DIMS, kT, COEF_UNIFORM, LINK_CONST>(b, total, iso, s);
+  else batch_dims<DIMS, kT, COEF_STEP, LINK_CONST>(b, total, iso, s);
+}
+
+ChunkShape shape_of(int dims, const int N[3], int steps) { return dims == 3 ? shape3d(N) : shape2d(N, steps); }
 
 }  // namespace
 
-int launch_fused2d_tb2(const FusedArgs<F32>& a, cudaStream_t s) {
-  const int c = a.hu.coef_mode, l = a.hu.link_mode;
-  if (c == COEF_UNIFORM && l == LINK_NONE) return launch2d_tb2<COEF_UNIFORM, LINK_NONE>(a, s);
-  if (c == COEF_STEP && l == LINK_NONE) return launch2d_tb2<COEF_STEP, LINK_NONE>(a, s);
-  if (c == COEF_UNIFORM && l == LINK_CONST) return launch2d_tb2<COEF_UNIFORM, LINK_CONST>(a, s);
-  if (c == COEF_STEP && l == LINK_CONST) return launch2d_tb2<COEF_STEP, LINK_CONST>(a, s);
-  if (c == COEF_TABLE && l == LINK_NONE) return launch2d_tb2<COEF_TABLE, LINK_NONE>(a, s);
-  if (c == COEF_SOFTCORE && l == LINK_NONE) return launch2d_tb2<COEF_SOFTCORE, LINK_NONE>(a, s);
-  if (c == COEF_SOFTCORR && l == LINK_NONE) return launch2d_tb2<COEF_SOFTCORR, LINK_NONE>(a, s);
-  return 0;
-}
+int launch_fused2d_two(const FusedArgs<F32>& a, cudaStream_t s) { return dispatch<2, 2>(a, s); }
 
-static ChunkShape shape_of(int dims, const int N[3], int two_step) {
-  return dims == 3 ? shape3d(N) : (two_step ? shape2d_tb2(N) : shape2d(N));
-}
-static long long items_of(const ChunkShape& g, int chunk) { return g.tiles * ((g.levels + chunk - 1) / chunk); }
+int fused_chunk(int dims, const int N[3], int steps) { return plan_chunk(shape_of(dims, N, steps)); }
 
-int fused_chunk_tb2(const int N[3]) { return plan_chunk(shape2d_tb2(N)); }
-
-long long fused_items_tb2(const int N[3], int chunk) { return items_of(shape2d_tb2(N), chunk); }
-
-void launch_fused2d_tb2_batch(const BatchArgs<F32>& b, long long total, int coef, int link, cudaStream_t s) {
-  if (coef == COEF_UNIFORM && link == LINK_NONE) return launch2d_tb2_batch<COEF_UNIFORM, LINK_NONE>(b, total, s);
-  if (coef == COEF_STEP && link == LINK_NONE) return launch2d_tb2_batch<COEF_STEP, LINK_NONE>(b, total, s);
-  if (coef == COEF_UNIFORM && link == LINK_CONST) return launch2d_tb2_batch<COEF_UNIFORM, LINK_CONST>(b, total, s);
-  return launch2d_tb2_batch<COEF_STEP, LINK_CONST>(b, total, s);
-}
-
-int fused_chunk(int dims, const int N[3]) { return plan_chunk(shape_of(dims, N, 0)); }
-
-int fused_candidates(int dims, const int N[3], int two_step, int* out, int max) {
-  const ChunkShape g = shape_of(dims, N, two_step);
+int fused_candidates(int dims, const int N[3], int steps, int* out, int max) {
+  const ChunkShape g = shape_of(dims, N, steps);
   return rank_chunks(g.tiles, g.levels, g.workers, g.min_chunk, g.restart, out, max);
 }
 
-long long fused_items(int dims, const int N[3], int chunk) { return items_of(shape_of(dims, N, 0), chunk); }
-
-template <>
-void launch_fused_batch<F32, 3>(const BatchArgs<F32>& b, long long total, int coef, int link,
-                                cudaStream_t s) {
-  if (coef == COEF_UNIFORM && link == LINK_NONE) return batch_dims<3, COEF_UNIFORM, LINK_NONE>(b, total, s);
-  if (coef == COEF_STEP && link == LINK_NONE) return batch_dims<3, COEF_STEP, LINK_NONE>(b, total, s);
-  if (coef == COEF_UNIFORM && link == LINK_CONST) return batch_dims<3, COEF_UNIFORM, LINK_CONST>(b, total, s);
-  return batch_dims<3, COEF_STEP, LINK_CONST>(b, total, s);
+long long fused_items(int dims, const int N[3], int steps, int chunk) {
+  const ChunkShape g = shape_of(dims, N, steps);
+  return g.tiles * ((g.levels + chunk - 1) / chunk);
 }
-template <>
-void launch_fused_batch<F32, 2>(const BatchArgs<F32>& b, long long total, int coef, int link,
-                                cudaStream_t s) {
-  if (coef == COEF_UNIFORM && link == LINK_NONE) return batch_dims<2, COEF_UNIFORM, LINK_NONE>(b, total, s);
-  if (coef == COEF_STEP && link == LINK_NONE) return batch_dims<2, COEF_STEP, LINK_NONE>(b, total, s);
-  if (coef == COEF_UNIFORM && link == LINK_CONST) return batch_dims<2, COEF_UNIFORM, LINK_CONST>(b, total, s);
-  return batch_dims<2, COEF_STEP, LINK_CONST>(b, total, s);
+
+void launch_fused_batch(const BatchArgs<F32>& b, int dims, int steps, long long total, int coef, int link, bool iso,
+                        cudaStream_t s) {
+  if (dims == 3) dispatch_batch<3, 1>(b, total, coef, link, iso, s);
+  else if (steps == 2) dispatch_batch<2, 2>(b, total, coef, link, iso, s);
+  else dispatch_batch<2, 1>(b, total, coef, link, iso, s);
 }
 
 template <>
 int launch_fused<F32, 3>(const FusedArgs<F32>& a, cudaStream_t s) {
-  return dispatch<3>(a, s);
+  return dispatch<3, 1>(a, s);
 }
 template <>
 int launch_fused<F32, 2>(const FusedArgs<F32>& a, cudaStream_t s) {
-  return dispatch<2>(a, s);
+  return dispatch<2, 1>(a, s);
 }
 
 }  // namespace dirac
