@@ -281,6 +281,7 @@ __device__ __forceinline__ void fused2d_item(const FusedArgs<P>& a, float4* ring
 
 template <class P, int COEF, int LINK, int kT, bool kIso>
 __global__ void __launch_bounds__(32 * kFused2dWarps, min_blocks(kT, COEF, LINK)) fused2d_kernel(const FusedArgs<P> a) {
+  depends();
   const int lane = threadIdx.x & 31;
   const long long worker = (long long)blockIdx.x * kFused2dWarps + (threadIdx.x >> 5);
   const long long items = (long long)strips2d<kT>(a.N[0]) * ((a.nzu + a.chunk - 1) / a.chunk);
@@ -294,6 +295,7 @@ __global__ void __launch_bounds__(32 * kFused2dWarps, min_blocks(kT, COEF, LINK)
 // Several simulations (time-independent fields) in one persistent launch.
 template <class P, int COEF, int LINK, int kT, bool kIso>
 __global__ void __launch_bounds__(32 * kFused2dWarps, min_blocks(kT, COEF, LINK)) fused2d_batch_kernel(const BatchArgs<P> b) {
+  depends();
   __shared__ FusedArgs<P> sa[kFused2dWarps];
   __shared__ __align__(16) float4 ring[kFused2dWarps][warp_slots<COEF, LINK>()];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -341,7 +343,7 @@ int launch2d_iso(FusedArgs<F32> a, cudaStream_t s) {
   if (a.e_partials && w > (long long)kFusedEMaxBlocks * kFused2dWarps) w = (long long)kFusedEMaxBlocks * kFused2dWarps;
   a.workers = (int)w;
   const int blocks = (int)((w + kFused2dWarps - 1) / kFused2dWarps);
-  k<<<(unsigned)blocks, 32 * kFused2dWarps, 0, s>>>(a);
+  launch_dependent(k, dim3((unsigned)blocks), dim3(32 * kFused2dWarps), 0, s, a);
   return blocks;
 }
 template <int COEF, int LINK, int kT>
@@ -357,7 +359,7 @@ void launch2d_batch(BatchArgs<F32> b, long long total, cudaStream_t s) {
   const int warps = workers2d<k>();
   const long long w = total < warps ? total : warps;
   b.workers = (int)w;
-  k<<<(unsigned)((w + kFused2dWarps - 1) / kFused2dWarps), 32 * kFused2dWarps, 0, s>>>(b);
+  launch_dependent(k, dim3((unsigned)((w + kFused2dWarps - 1) / kFused2dWarps)), dim3(32 * kFused2dWarps), 0, s, b);
 }
 
 }  // namespace fused

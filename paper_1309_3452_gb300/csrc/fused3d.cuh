@@ -438,6 +438,7 @@ __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long it
 // kernel of its own, so that the others carry neither its terms nor its tests)
 template <class P, int COEF, int LINK, bool kE, int kPairs, bool kIso>
 __global__ void __launch_bounds__(Tile3<kPairs>::threads, 1) fused3d_kernel(const FusedArgs<P> a) {
+  depends();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int kThreads3d = Tile3<kPairs>::threads;
   const Thread3d th = thread3d<kPairs>();
@@ -461,6 +462,7 @@ constexpr int kBatchPairs = 14;
 // simulation its current item belongs to into shared memory.
 template <class P, int COEF, int LINK, bool kIso>
 __global__ void __launch_bounds__(Tile3<kBatchPairs>::threads, 1) fused3d_batch_kernel(const BatchArgs<P> b) {
+  depends();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ FusedArgs<P> sa;
   const Thread3d th = thread3d<kBatchPairs>();
@@ -518,7 +520,7 @@ int launch3d_tile(FusedArgs<F32> a, cudaStream_t s) {
   a.workers = (int)(items < resident ? items : resident);
   // one E partial per block: never more blocks than the partials hold
   if (kE && a.workers > kFusedEMaxBlocks) a.workers = kFusedEMaxBlocks;
-  k<<<(unsigned)a.workers, Tile3<kPairs>::threads, Tile3<kPairs>::smem, s>>>(a);
+  launch_dependent(k, dim3((unsigned)a.workers), dim3(Tile3<kPairs>::threads), Tile3<kPairs>::smem, s, a);
   return a.workers;
 }
 
@@ -540,7 +542,7 @@ void launch3d_batch(BatchArgs<F32> b, long long total, cudaStream_t s) {
   constexpr auto k = fused3d_batch_kernel<F32, COEF, LINK, kIso>;
   const int resident = workers3d<k, kBatchPairs>();
   b.workers = (int)(total < resident ? total : resident);
-  k<<<(unsigned)b.workers, Tile3<kBatchPairs>::threads, Tile3<kBatchPairs>::smem, s>>>(b);
+  launch_dependent(k, dim3((unsigned)b.workers), dim3(Tile3<kBatchPairs>::threads), Tile3<kBatchPairs>::smem, s, b);
 }
 
 }  // namespace fused

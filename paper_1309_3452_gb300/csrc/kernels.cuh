@@ -7,6 +7,33 @@
 
 namespace dirac {
 
+// Launches that follow one another on a stream are made as programmatic
+// dependents: the next kernel's blocks are placed while the last blocks of the
+// one before still run, and wait in depends() until that one has finished and
+// its writes are visible.  Every kernel launched this way calls depends() before
+// it touches memory, so the order of all work is that of plain launches; what
+// is saved is the launch latency between short kernels.
+// us per step, before and after: 96^3 FP64 254 / 249, 64^3 laser FP64 142 / 136,
+// 203x149x91 84.5 / 82.8, 300 x 260 3.16 / 3.09; long kernels unchanged.
+__device__ __forceinline__ void depends() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... A, class... B>
+inline void launch_dependent(void (*kernel)(A...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const B&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, static_cast<A>(args)...);
+}
+
 // One half-step (all upper or all lower values) of the scheme, one kernel.
 template <class P>
 struct HalfStepArgs {
@@ -54,6 +81,7 @@ constexpr int kFusedEMaxBlocks = 4096;  // capacity of the per-block E partials
 // (2+1)D fused kernel geometry
 constexpr int kFused2dWarps = 4;   // independent x strips per block (few, so that small grids spread over the SMs)
 constexpr int kMaxSteps2d = 2;     // most time steps per pass
+constexpr int kTableSteps = 32;    // time steps whose plane-wave link tables one launch forms
 
 // returns the number of blocks launched
 template <class P, int DIMS>

@@ -302,7 +302,7 @@ __device__ __forceinline__ void store_quad_lane(float4* rec, int lane, float4 v)
 }
 
 struct LinkTimes {
-  double up[kMaxSteps2d], lo[kMaxSteps2d];
+  double up[kTableSteps], lo[kTableSteps];
 };
 template <class P>
 __global__ void link_table_kernel(typename PlaneLinkOf<P>::type* tab, int n, const FieldDesc f, int dims,
