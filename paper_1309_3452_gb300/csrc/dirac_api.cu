@@ -49,7 +49,7 @@ struct dirac_sim {
   F64::Coef* c_tab = nullptr; // COEF_TABLE, FP64: alpha and gamma per site (plane-major, pstride)
   unsigned* sc_corr = nullptr; // COEF_SOFTCORR: one 32-bit correction word per value
   double* Alink = nullptr;    // link integrals x q: 2 dims slots (up, down link per axis) of np * pstride
-  F32::Link* larr = nullptr;  // LINK_TABLE: link factors, same slots, FP32 hi + lo
+  void* larr = nullptr;       // LINK_TABLE, LINK_UP: link factors (F32::Link, FP64: F64::Link)
   double* partials = nullptr;
   double* sums_dev = nullptr;
   double* sums_host = nullptr; // pinned
@@ -305,7 +305,7 @@ static HalfFields<P> half_fields(const dirac_sim* s, bool upper, double t) {
   h.c_ps = s->pstride;
   if (s->fused) {
     h.bq = s->b_tab;
-    h.lq = s->link_mode == LINK_TABLE ? reinterpret_cast<const float4*>(s->larr) : nullptr;
+    h.lq = s->link_mode == LINK_TABLE ? static_cast<const float4*>(s->larr) : nullptr;
     h.q_ps = s->pstride;
   }
   split(rx, h.rx_hi, h.rx_lo);
@@ -325,8 +325,8 @@ static HalfFields<P> half_fields(const dirac_sim* s, bool upper, double t) {
     }
     h.sc_corr = s->sc_corr;
   }
-  if (s->link_mode == LINK_TABLE && !s->fused) {
-    h.larr = reinterpret_cast<const typename P::Link*>(s->larr);
+  if ((s->link_mode == LINK_TABLE && !s->fused) || s->link_mode == LINK_UP) {
+    h.larr = static_cast<const typename P::Link*>(s->larr);
     h.larr_n = (long long)s->np * s->pstride;
     h.larr_ps = s->pstride;
   }
@@ -573,7 +573,11 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
   // tabulated once for the FP32 kernels instead of a sincos per link and step
   const bool moving = (f.Apw_amp != 0.0 && f.Apw_omega != 0.0) ||
                       (alinks && f.Alink_amp != 0.0 && f.Alink_omega != 0.0);
-  if (precision == DIRAC_FP32 && s->link_mode == LINK_GENERAL && !moving) s->link_mode = LINK_TABLE;
+  // (FP64: where it is given by its link integrals alone and the memory allows it)
+  if (s->link_mode == LINK_GENERAL && !moving) {
+    if (precision == DIRAC_FP32) s->link_mode = LINK_TABLE;
+    else if (alinks && f.Apw_amp == 0.0) s->link_mode = LINK_UP;
+  }
 
   auto cleanup_fail = [&](dirac_status st) {
     std::string msg = s->err;
@@ -626,15 +630,37 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
     cudaFree(raw);
     if (e != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "link integral table"));
   }
-  if (s->link_mode == LINK_TABLE) {  // after the link integrals: the phases include them
-    const size_t tb = (size_t)2 * dims * s->np * s->pstride * sizeof(F32::Link);
-    if ((e = cudaMalloc(&s->larr, tb)) != cudaSuccess)
-      return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link factor table)"));
-    if ((e = cudaMemsetAsync(s->larr, 0, tb, s->stream)) != cudaSuccess)
-      return cleanup_fail(cuda_fail(s, e, "cudaMemsetAsync(link factor table)"));
-    launch_link_factor_table(s->larr, field_desc(s), dims, s->N, s->pstride, s->fused, s->stream);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "link factor table"));
-    s->launches += 1;
+  if (s->link_mode == LINK_TABLE || s->link_mode == LINK_UP) {  // after the link integrals: the phases include them
+    const int dirs = s->link_mode == LINK_UP ? 1 : 2;
+    const size_t tb = (size_t)dirs * dims * s->np * s->pstride * sizeof(F32::Link);
+    static_assert(sizeof(F32::Link) == sizeof(F64::Link), "one size for both precisions");
+    if (precision == DIRAC_FP64) {  // where the table leaves as much device memory as it takes, else per site
+      size_t mem_free = 0, mem_total = 0;
+      if ((e = cudaMemGetInfo(&mem_free, &mem_total)) != cudaSuccess)
+        return cleanup_fail(cuda_fail(s, e, "cudaMemGetInfo"));
+      e = tb <= mem_free / 2 ? cudaMalloc(&s->larr, tb) : cudaErrorMemoryAllocation;
+      if (e == cudaErrorMemoryAllocation) {
+        s->larr = nullptr;
+        cudaGetLastError();  // not an error of this simulation
+        s->link_mode = LINK_GENERAL;
+        e = cudaSuccess;
+      }
+    } else {
+      e = cudaMalloc(&s->larr, tb);
+    }
+    if (e != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link factor table)"));
+    if (s->larr) {
+      if ((e = cudaMemsetAsync(s->larr, 0, tb, s->stream)) != cudaSuccess)
+        return cleanup_fail(cuda_fail(s, e, "cudaMemsetAsync(link factor table)"));
+      if (precision == DIRAC_FP64)
+        launch_link_factor_table<F64>(static_cast<F64::Link*>(s->larr), field_desc(s), dims, s->N, s->pstride, 0, dirs,
+                                      s->stream);
+      else
+        launch_link_factor_table<F32>(static_cast<F32::Link*>(s->larr), field_desc(s), dims, s->N, s->pstride,
+                                      s->fused, dirs, s->stream);
+      if ((e = cudaGetLastError()) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "link factor table"));
+      s->launches += 1;
+    }
   }
   if (s->coef_mode == COEF_SOFTCORE || s->coef_mode == COEF_SOFTCORR) {
     std::vector<float2> sq;
@@ -1416,7 +1442,11 @@ static dirac_status observe_launch(dirac_sim* s, int dens_axis, int dens_X, doub
     a.wave = s->wave;
     a.wave_axis = s->ltab_axis;
   }
-  if (s->link_mode == LINK_TABLE && s->fused) a.lq = reinterpret_cast<const float4*>(s->larr);
+  if (s->link_mode == LINK_TABLE && s->fused) a.lq = static_cast<const float4*>(s->larr);
+  if (s->link_mode == LINK_UP) {
+    a.larr = static_cast<const typename P::Link*>(s->larr);
+    a.larr_n = (long long)s->np * s->pstride;
+  }
   a.dens_axis = dens_axis;
   a.dens_X = dens_X;
   a.partials = s->partials;
@@ -1651,7 +1681,7 @@ extern "C" dirac_status dirac_check(dirac_sim* s, double tol, dirac_check_report
   // bounds of the functional as a quadratic form
   double lo = 0.0, hi = 0.0;
   const int general_A = s->link_mode == LINK_GENERAL || s->link_mode == LINK_PLANE ||
-                        s->link_mode == LINK_TABLE;
+                        s->link_mode == LINK_TABLE || s->link_mode == LINK_UP;
   dirac_functional_bounds(s->dims, s->dx, s->dt, general_A, &lo, &hi);
   r.lower = 0.0;
   r.upper = INFINITY;

@@ -131,6 +131,8 @@ struct ObsArgs {
   const void* wave;
   int wave_axis;
   const float4* lq;
+  const typename P::Link* larr;  // LINK_UP: the up links, [axis * larr_n + plane * pstride + cell]
+  long long larr_n;
   int dens_axis, dens_X;    // partial density: half-lattice index >= dens_X along axis
   double* partials;         // [gridDim.x][5]
   int zlo, nzu, zorg, Nzg;  // levels summed along the marching axis and their global position, as in FusedArgs
@@ -178,12 +180,13 @@ void launch_softcore_corr(unsigned* out, const HalfFields<F32>& hu, const HalfFi
 void launch_link_integral_table(double* out, const double* raw, int dims, const int N[3], long long pstride,
                                 double q, cudaStream_t s);
 
-// LINK_TABLE: exp(-i phi) of every value's up link (slot 2a) and down link
-// (slot 2a+1) of a time-independent vector potential, FP32 hi + lo pairs:
-// out[slot * P * pstride + plane * pstride + cell], or (quads) as the quad
-// records of quad.cuh, slot by slot
-void launch_link_factor_table(F32::Link* out, const FieldDesc& f, int dims, const int N[3], long long pstride,
-                              int quads, cudaStream_t s);
+// exp(-i phi) of every value's links of a time-independent vector potential:
+// out[slot * P * pstride + plane * pstride + cell], or (quads, F32) the quad
+// records of quad.cuh, slot by slot.  dirs = 2 (LINK_TABLE): slot 2a the up
+// link along axis a, 2a+1 the down link; dirs = 1 (LINK_UP): slot a the up link
+template <class P>
+void launch_link_factor_table(typename P::Link* out, const FieldDesc& f, int dims, const int N[3], long long pstride,
+                              int quads, int dirs, cudaStream_t s);
 
 // measured FP64 FMA rate of the current device (TFLOP/s), < 0 on a CUDA failure
 double measure_fp64_fma_tflops();

@@ -214,6 +214,13 @@ __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
               up = link_mul(a.L[ax], up);
               dn = link_mulc(a.L[ax], dn);
             }
+            if constexpr (kLink == LINK_UP) {
+              const long long below = plane_off<DIMS>(plane, ax) ? cell
+                                      : (ax == 0 ? cell + dxm : (ax == 1 ? cell + dym : cell + (z == 0 ? nxy * Nz - nxy : -nxy)));
+              const typename P::Link* t = a.larr + ax * a.larr_n;
+              up = link_mul(up_link<P>(t + (plane * a.pstride + cell)), up);
+              dn = link_mulc(up_link<P>(t + (partner<DIMS>(plane, ax) * a.pstride + below)), dn);
+            }
             if constexpr (kLink == LINK_TABLE && kQuads) {
               const float4* t = a.lq + 2 * ((long long)(2 * ax * nc + c) * a.pstride + cell);
               const float4 u = quad_lane(t, l), d = quad_lane(t + 2 * nc * a.pstride, l);
@@ -438,11 +445,12 @@ __global__ void link_integral_table_kernel(double* __restrict__ out, const doubl
 
 // LINK_TABLE: the link factors exp(-i phi) of every value of a time-independent
 // vector potential, phi from the same FP64 function as the per-site path
-// (dir 0: the value's up link; dir 1: the link from its lower neighbour)
-template <int DIMS>
-__global__ void link_factor_table_kernel(F32::Link* __restrict__ out, const FieldDesc f, int N0, int N1, int N2,
-                                         long long pstride, int quads) {
-  const int plane = blockIdx.y, slot = blockIdx.z, axis = slot >> 1, dir = (slot & 1) ? -1 : 1;
+// (slot 2 axis: the value's up link; 2 axis + 1: the link from its lower
+// neighbour); LINK_UP (dirs == 1): the up links alone, slot = axis
+template <class P, int DIMS>
+__global__ void link_factor_table_kernel(typename P::Link* __restrict__ out, const FieldDesc f, int N0, int N1, int N2,
+                                         long long pstride, int quads, int dirs) {
+  const int plane = blockIdx.y, slot = blockIdx.z, axis = slot / dirs, dir = slot % dirs ? -1 : 1;
   const long long ncell = (long long)N0 * N1 * N2;
   const long long n = (long long)nplanes<DIMS>() * pstride;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
@@ -451,11 +459,15 @@ __global__ void link_factor_table_kernel(F32::Link* __restrict__ out, const Fiel
     const long long H[3] = {2 * x + plane_off<DIMS>(plane, 0), 2 * y + plane_off<DIMS>(plane, 1),
                             DIMS == 3 ? 2 * z + plane_off<DIMS>(plane, 2) : 0};
     const double phi = link_phase_site(f, DIMS, H, axis, dir, 0.0, plane, c);
-    const F32::Link L = link_from(phi, (F32*)nullptr);
-    if (quads)  // the quads of slot, component: 2 * ((slot * components + component) * pstride + cell)
-      store_quad_lane(reinterpret_cast<float4*>(out) + slot * n + 2 * ((plane >> 1) * pstride + c), plane & 1,
-                      make_float4(L.hi.x, L.hi.y, L.lo.x, L.lo.y));
-    else out[slot * n + plane * pstride + c] = L;
+    const typename P::Link L = link_from(phi, (P*)nullptr);
+    if constexpr (sizeof(typename P::real) == 4) {
+      if (quads) {  // the quads of slot, component: 2 * ((slot * components + component) * pstride + cell)
+        store_quad_lane(reinterpret_cast<float4*>(out) + slot * n + 2 * ((plane >> 1) * pstride + c), plane & 1,
+                        make_float4(L.hi.x, L.hi.y, L.lo.x, L.lo.y));
+        continue;
+      }
+    }
+    out[slot * n + plane * pstride + c] = L;
   }
 }
 
@@ -595,6 +607,8 @@ static int launch_observables_link(const ObsArgs<P>& a, int blocks, cudaStream_t
   if (l == LINK_NONE) return launch_observables_path<P, DIMS, kQuads, LINK_NONE, kDens>(a, blocks, s);
   if (l == LINK_CONST) return launch_observables_path<P, DIMS, kQuads, LINK_CONST, kDens>(a, blocks, s);
   if (l == LINK_PLANE && a.wave) return launch_observables_path<P, DIMS, kQuads, LINK_PLANE, kDens>(a, blocks, s);
+  if constexpr (sizeof(typename P::real) == 8)
+    if (l == LINK_UP) return launch_observables_path<P, DIMS, kQuads, LINK_UP, kDens>(a, blocks, s);
   if (kQuads && l == LINK_TABLE)
     return launch_observables_path<P, DIMS, kQuads, kQuads ? LINK_TABLE : LINK_GENERAL, kDens>(a, blocks, s);
   return launch_observables_path<P, DIMS, kQuads, LINK_GENERAL, kDens>(a, blocks, s);
@@ -677,17 +691,22 @@ void launch_link_integral_table(double* out, const double* raw, int dims, const 
     link_integral_table_kernel<2><<<grid, 256, 0, s>>>(out, raw, N[0], N[1], 1, pstride, q);
 }
 
-void launch_link_factor_table(F32::Link* out, const FieldDesc& f, int dims, const int N[3], long long pstride,
-                              int quads, cudaStream_t s) {
+template <class P>
+void launch_link_factor_table(typename P::Link* out, const FieldDesc& f, int dims, const int N[3], long long pstride,
+                              int quads, int dirs, cudaStream_t s) {
   const long long ncell = (long long)N[0] * N[1] * (dims == 3 ? N[2] : 1);
   long long bx = (ncell + 255) / 256;
   if (bx > 152 * 16) bx = 152 * 16;
-  const dim3 grid((unsigned)bx, dims == 3 ? 8 : 4, 2 * dims);
+  const dim3 grid((unsigned)bx, dims == 3 ? 8 : 4, dirs * dims);
   if (dims == 3)
-    link_factor_table_kernel<3><<<grid, 256, 0, s>>>(out, f, N[0], N[1], N[2], pstride, quads);
+    link_factor_table_kernel<P, 3><<<grid, 256, 0, s>>>(out, f, N[0], N[1], N[2], pstride, quads, dirs);
   else
-    link_factor_table_kernel<2><<<grid, 256, 0, s>>>(out, f, N[0], N[1], 1, pstride, quads);
+    link_factor_table_kernel<P, 2><<<grid, 256, 0, s>>>(out, f, N[0], N[1], 1, pstride, quads, dirs);
 }
+template void launch_link_factor_table<F32>(F32::Link*, const FieldDesc&, int, const int[3], long long, int, int,
+                                            cudaStream_t);
+template void launch_link_factor_table<F64>(F64::Link*, const FieldDesc&, int, const int[3], long long, int, int,
+                                            cudaStream_t);
 
 void launch_finish_sums2(const double* partials, int nblocks, double* out, cudaStream_t s) {
   finish_sums_kernel<2><<<1, 64, 0, s>>>(partials, nblocks, out);

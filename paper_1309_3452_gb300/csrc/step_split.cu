@@ -74,6 +74,9 @@ void launch_one(const HalfStepArgs<P>& a, cudaStream_t s) {
   else if (!f32 && c == COEF_UNIFORM && l == LINK_CONST) HALF_STEP(COEF_UNIFORM, f32 ? LINK_NONE : LINK_CONST);
   else if (!f32 && c == COEF_STEP && l == LINK_CONST) HALF_STEP(COEF_STEP, f32 ? LINK_NONE : LINK_CONST);
   else if (!f32 && c == COEF_TABLE && l == LINK_CONST) HALF_STEP(COEF_TABLE, f32 ? LINK_NONE : LINK_CONST);
+  else if (!f32 && c == COEF_UNIFORM && l == LINK_UP) HALF_STEP(COEF_UNIFORM, f32 ? LINK_NONE : LINK_UP);
+  else if (!f32 && c == COEF_STEP && l == LINK_UP) HALF_STEP(COEF_STEP, f32 ? LINK_NONE : LINK_UP);
+  else if (!f32 && c == COEF_TABLE && l == LINK_UP) HALF_STEP(COEF_TABLE, f32 ? LINK_NONE : LINK_UP);
   else HALF_STEP(kAnyMode, kAnyMode);
 #undef HALF_STEP
 }
