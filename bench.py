@@ -189,8 +189,9 @@ class Clocks:
 
 KERNEL_SOURCES = {  # the files that determine each timed kernel's code
     "step_fp32": ["step_fused.cu", "fused_common.cuh", "fused3d.cuh", "fused3d_basic.cu", "fused3d_fields.cu",
-                  "fused3d_links.cu", "fused3d_wave.cu", "fused2d.cu", "quad.cuh", "common.cuh", "kernels.cuh"],
-    "step_fp64": ["step_split.cu", "common.cuh", "kernels.cuh"],
+                  "fused3d_links.cu", "fused3d_wave.cu", "fused2d.cuh", "fused2d_basic.cu", "fused2d_fields.cu",
+                  "fused2d_wave.cu", "quad.cuh", "common.cuh", "kernels.cuh"],
+    "step_fp64": ["step_split.cu", "fused_common.cuh", "common.cuh", "kernels.cuh"],
 }
 
 

@@ -267,7 +267,7 @@ long long dirac_kernel_launches(const dirac_sim* sim);
  * order and may differ in the last bits.
  *   chunk       z levels ((3+1)D) or y rows ((2+1)D) per work item of the
  *               one-step kernel; 0 = the built-in rule
- *   two_step    (2+1)D: 1 = four or two time steps per pass whenever the field
+ *   two_step    (2+1)D: 1 = two time steps per pass whenever the field
  *               path allows it (the default), 0 = one step per pass
  *   chunk2      rows per work item of those passes; 0 = the rule
  *   us_per_step time per step that dirac_autotune measured for this plan
