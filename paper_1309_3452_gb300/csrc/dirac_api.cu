@@ -45,6 +45,8 @@ struct dirac_sim {
   double* Vstatic = nullptr;  // one real per site (plane-major, pstride)
   int vstatic = 0;            // the caller gave a static array (which a table may have replaced)
   float4* b_tab = nullptr;    // COEF_TABLE: b = 1/(1 + i theta) per site as hi + lo (plane-major, pstride)
+  unsigned* b_map = nullptr;  // fused kernels: the cells' classes in b_tab, and a cell of each (HalfFields::b_map)
+  long long b_ps = 0;         // classes (b_tab's records per component)
   float2* sc_sq = nullptr;    // COEF_SOFTCORE/CORR: (X dx_a/2 - c_a)^2 per axis and half-lattice index, hi + lo
   F64::Coef* c_tab = nullptr; // COEF_TABLE, FP64: alpha and gamma per site (plane-major, pstride)
   unsigned* sc_corr = nullptr; // COEF_SOFTCORR: one 32-bit correction word per value
@@ -237,6 +239,7 @@ static void softcore_tables(const dirac_sim* s, std::vector<float2>& out) {
   }
 }
 
+static bool per_site_path(const dirac_sim* s);
 static FieldDesc field_desc(const dirac_sim* s) {
   FieldDesc d;
   std::memset(&d, 0, sizeof(d));
@@ -276,6 +279,42 @@ static FieldDesc field_desc(const dirac_sim* s) {
   return d;
 }
 
+// The classes of cells with the same tabulated coefficients (HalfFields::b_map):
+// out = the classes' parts by x, y and z, then one cell coordinate of every
+// class along x, y and z; n the classes per axis.  Not shared: every cell its
+// own.  Shared (V0, a uniform imaginary part, absorbing layers and a Klein step,
+// nothing else): along an axis the cells with neither of their two half-lattice
+// points in a layer (potential_imag_at's test) differ only by their points'
+// sides of the step.
+static void coef_classes(const dirac_sim* s, bool shared, std::vector<unsigned>& out, int (&n)[3]) {
+  const FieldDesc f = field_desc(s);
+  std::vector<unsigned> rep;
+  unsigned stride = 1;
+  out.clear();
+  for (int a = 0; a < 3; ++a) {
+    n[a] = 0;
+    int inside[4] = {-1, -1, -1, -1};  // class by the two points' sides
+    for (int i = 0; i < s->N[a]; ++i) {
+      bool in_layer = false;
+      int sides = 0;
+      for (int p = 0; p < 2; ++p) {
+        const double x = (double)(2LL * i + p) * f.dx[a] * 0.5;
+        if (a < s->dims && ((f.abs_axes >> a) & 1) && std::fmin(x, f.L[a] - x) < f.abs_width) in_layer = true;
+        if (f.step_axis == a && 2LL * i + p >= f.step_X) sides |= 1 << p;
+      }
+      int c = shared && !in_layer ? inside[sides] : -1;
+      if (c < 0) {
+        c = n[a]++;
+        rep.push_back((unsigned)i);
+        if (shared && !in_layer) inside[sides] = c;
+      }
+      out.push_back(stride * (unsigned)c);
+    }
+    stride *= (unsigned)n[a];
+  }
+  out.insert(out.end(), rep.begin(), rep.end());
+}
+
 template <class P>
 static void plane_ptrs(dirac_sim* s, typename P::cplx* (&pl)[8]) {
   auto* base = static_cast<typename P::cplx*>(s->state);
@@ -305,6 +344,8 @@ static HalfFields<P> half_fields(const dirac_sim* s, bool upper, double t) {
   h.c_ps = s->pstride;
   if (s->fused) {
     h.bq = s->b_tab;
+    h.b_map = s->b_map;
+    h.b_ps = s->b_ps;
     h.lq = s->link_mode == LINK_TABLE ? static_cast<const float4*>(s->larr) : nullptr;
     h.q_ps = s->pstride;
   }
@@ -720,9 +761,28 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
     }
   }
   if (s->coef_mode == COEF_TABLE && !s->c_tab) {
-    if ((e = cudaMalloc(&s->b_tab, (size_t)s->np * s->pstride * sizeof(float4))) != cudaSuccess)
+    s->b_ps = s->pstride;
+    int classes[3] = {s->N[0], s->N[1], s->N[2]};
+    const int* rep = nullptr;
+    if (s->fused) {
+      std::vector<unsigned> map;
+      // (the run-time kernel, which such a vector potential or a plane wave in
+      // (3+1)D other than LINK_PLANE_ZX takes, reads the table by site)
+      const bool by_site = per_site_path(s) ||
+                           (dims == 3 && s->link_mode == LINK_PLANE && (s->ltab_axis != 2 || f.Apw_pol != 0));
+      const bool shared = layers && !vstatic && f.sc_Z == 0.0 && !slab.on && !by_site;
+      coef_classes(s, shared, map, classes);
+      if (shared) s->b_ps = (long long)classes[0] * classes[1] * classes[2];
+      if ((e = cudaMalloc(&s->b_map, map.size() * sizeof(unsigned))) != cudaSuccess)
+        return cleanup_fail(cuda_fail(s, e, "cudaMalloc(coefficient classes)"));
+      // synchronous: the host vector goes out of scope
+      if ((e = cudaMemcpy(s->b_map, map.data(), map.size() * sizeof(unsigned), cudaMemcpyHostToDevice)) != cudaSuccess)
+        return cleanup_fail(cuda_fail(s, e, "cudaMemcpy(coefficient classes)"));
+      if (shared) rep = reinterpret_cast<const int*>(s->b_map) + s->N[0] + s->N[1] + s->N[2];
+    }
+    if ((e = cudaMalloc(&s->b_tab, (size_t)s->np * s->b_ps * sizeof(float4))) != cudaSuccess)
       return cleanup_fail(cuda_fail(s, e, "cudaMalloc(coefficient table)"));
-    launch_coef_table(s->b_tab, field_desc(s), dims, s->N, s->pstride, s->fused, s->stream);
+    launch_coef_table(s->b_tab, field_desc(s), dims, classes, s->b_ps, s->fused, rep, s->stream);
     if ((e = cudaGetLastError()) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "coefficient table"));
     s->launches += 1;
   }
@@ -774,6 +834,7 @@ extern "C" void dirac_destroy(dirac_sim* s) {
   cudaFree(s->staging);
   cudaFree(s->Vstatic);
   cudaFree(s->b_tab);
+  cudaFree(s->b_map);
   cudaFree(s->c_tab);
   cudaFree(s->sc_sq);
   cudaFree(s->sc_corr);

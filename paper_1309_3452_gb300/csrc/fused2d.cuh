@@ -70,7 +70,7 @@ struct WaveAt {
 // v1 (0,1).
 template <class P, int COEF, int LINK, bool kIso>
 __device__ __forceinline__ void row2d(const FusedArgs<P>& a, bool iso, int hx, int yk, int yn, long long ok,
-                                      long long on, const Quad& U, const Quad& V, const Quad& Vn, float2 nU0,
+                                      long long on, long long ck, long long cn, const Quad& U, const Quad& V, const Quad& Vn, float2 nU0,
                                       float2 nU1, const float4* lanes, const WaveAt& w, Quad& nU, Quad& nV, Quad* S) {
   const float2 v0n = qlane(Vn, 0), v1n = qlane(Vn, 1), v0 = qlane(V, 0), v1 = qlane(V, 1);
   {  // u0(k+1) from v0(k+1) (x), v1(k+1), v1(k) (y); u1(k) from v1(k) (x), v0(k+1), v0(k) (y)
@@ -80,7 +80,7 @@ __device__ __forceinline__ void row2d(const FusedArgs<P>& a, bool iso, int hx, i
     up[1] = mkquad(v1n, v0n);
     dn[1] = mkquad(v1, v0);
     const int H0[3] = {hx, 2 * yn, 0}, H1[3] = {hx + 1, 2 * yk + 1, 0};
-    nU = quad_update<2, COEF, LINK, false, kIso>(a.hu, a.f, iso, a.ry, a.rz, 0, U, up, dn, H0, H1, on, ok, a.pstride,
+    nU = quad_update<2, COEF, LINK, false, kIso>(a.hu, a.f, iso, a.ry, a.rz, 0, U, up, dn, H0, H1, on, ok, cn, ck, a.pstride,
                                            nullptr, nullptr, nullptr, a.N, lanes, w.u0, w.u1);
   }
   {  // v0(k) from u0(k) (x), u1(k), u1(k-1) (y); v1(k) from u1(k) (x), u0(k+1), u0(k) (y)
@@ -91,7 +91,7 @@ __device__ __forceinline__ void row2d(const FusedArgs<P>& a, bool iso, int hx, i
     up[1] = mkquad(u1k, u0n);
     dn[1] = mkquad(nU1, nU0);
     const int H0[3] = {hx + 1, 2 * yk, 0}, H1[3] = {hx, 2 * yk + 1, 0};
-    nV = quad_update<2, COEF, LINK, true, kIso>(a.hl, a.f, iso, a.ry, a.rz, 1, V, up, dn, H0, H1, ok, ok, a.pstride, S,
+    nV = quad_update<2, COEF, LINK, true, kIso>(a.hl, a.f, iso, a.ry, a.rz, 1, V, up, dn, H0, H1, ok, ok, ck, ck, a.pstride, S,
                                           nullptr, nullptr, a.N, lanes + 128, w.v0, w.v1);
   }
 }
@@ -127,6 +127,10 @@ __device__ __forceinline__ void march2d(const FusedArgs<P>& a, float4* ring, int
   const int hx = 2 * x;
   using Off = unsigned;  // (a level has fewer than 2^31 cells)
   auto off = [&](int k) { return (Off)stored(k) * (Off)Nx + (Off)x; };
+  auto class_of = [&](int k) -> long long {  // (COEF_TABLE)
+    if constexpr (COEF == COEF_TABLE) return __ldg(a.hu.b_map + x) + __ldg(a.hu.b_map + Nx + stored(k));
+    else return 0;
+  };
   const float4* lanes = ring + kRing * 64 + lane;  // (COEF_LANES)
   // LINK_PLANE: the factors from the steps' tables, [stage][half][parity of the
   // half-lattice coordinate].  A wave along y has the same ones for the whole
@@ -204,7 +208,7 @@ __device__ __forceinline__ void march2d(const FusedArgs<P>& a, float4* ring, int
     constexpr int next = s + 1 < kT ? s + 1 : 0;
     const int r = k - 2 * s;
     Quad nU, nV;
-    row2d<P, COEF, LINK, kIso>(a, iso, hx, gy(r), gy(r + 1), off(r), off(r + 1), U[s], V[s], Vn[s], nU0[s], nU1[s],
+    row2d<P, COEF, LINK, kIso>(a, iso, hx, gy(r), gy(r + 1), off(r), off(r + 1), class_of(r), class_of(r + 1), U[s], V[s], Vn[s], nU0[s], nU1[s],
                                lanes, wave_at(s, r), nU, nV, s == kT - 1 ? &oS : nullptr);
     if constexpr (s == kT - 1) {
       oU = mkquad(nU0[s], qlane(nU, 1));  // the row's new u0 (formed one row earlier) and u1

@@ -211,6 +211,15 @@ __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long it
       sRxy[c][1][threadIdx.x] = make_float4(a10.x, a01.x, a10.y, a01.y);
     }
   }
+  // COEF_TABLE: the x-y part of the two cells' classes
+  constexpr bool kTab = COEF == COEF_TABLE;
+  const unsigned* class_z = kTab ? a.hu.b_map + Nx + Ny : nullptr;
+  Off cls0 = 0, cls1 = 0;
+  if constexpr (kTab) {
+    const Off cx = __ldg(a.hu.b_map + x);
+    cls0 = cx + __ldg(a.hu.b_map + Nx + y0);
+    cls1 = cx + __ldg(a.hu.b_map + Nx + y1);
+  }
   // Per-level field constants, the same for the whole block, staged in
   // shared memory by threads 0..6 with copies that bypass the registers,
   // double-buffered by level parity (level k's copies are issued after the
@@ -279,7 +288,8 @@ __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long it
   };
   // both values of component comp (0 A, 1 B, 2 C, 3 D) of one cell: F the old
   // record, q, xt, ym1, yp0 the partner component around it (xy_neighbours), zu
-  // and zd the z partner's records, Z the level's half-lattice z, site the cell
+  // and zd the z partner's records, Z the level's half-lattice z, site the cell,
+  // rec its class (COEF_TABLE) or the cell of the level's correction record
   auto update = [&](auto comp_c, int cell, const Quad& F, const Quad& q, const float* xt, float2 ym1, float2 yp0,
                     const Quad& zu, const Quad& zd, int Z, float2 zq, Off site, Off rec, Quad* S, const PL* lk) {
     constexpr int comp = decltype(comp_c)::value;
@@ -293,7 +303,7 @@ __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long it
     dn[2] = zd;
     SoftB2 b;
     if constexpr (kSoft) b = pair_b(h, cell, xy, zq, H0, H1, rec, 2 * comp);
-    return quad_update<3, COEF, LINK, true, kIso>(h, a.f, iso, a.ry, a.rz, comp, F, up, dn, H0, H1, site, site, a.pstride, S,
+    return quad_update<3, COEF, LINK, true, kIso>(h, a.f, iso, a.ry, a.rz, comp, F, up, dn, H0, H1, site, site, rec, rec, a.pstride, S,
                                             kSoft ? &b : nullptr, lk, a.N);
   };
 
@@ -332,12 +342,20 @@ __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long it
   using IC = std::integral_constant<int, 2>;
   using ID = std::integral_constant<int, 3>;
 
+  Off class_n = 0;  // COEF_TABLE: the z part of the classes of level k + 1
+  if constexpr (kTab) class_n = __ldg(class_z + (z0 ? z0 - 1 : Nz - 1));
 #pragma unroll 1
   for (int k = z0 - 1; k < z1; ++k) {
     const int zk = k < 0 ? k + Nz : k;
     const int zn = k + 1 >= Nz ? k + 1 - Nz : k + 1;
     const Off ok0 = (Off)zk * nxy + cxy0, on0 = (Off)zn * nxy + cxy0;
     const Off ok1 = (Off)zk * nxy + cxy1, on1 = (Off)zn * nxy + cxy1;
+    Off rk0 = ok0, rn0 = ok0, rk1 = ok1, rn1 = ok1;
+    if constexpr (kTab) {
+      rk0 = class_n + cls0, rk1 = class_n + cls1;
+      class_n = __ldg(class_z + zn);
+      rn0 = class_n + cls0, rn1 = class_n + cls1;
+    }
     const int pk = k & 1;
     const int Zk = 2 * gz(k), Zn = 2 * gz(k + 1);  // half-lattice z of levels k, k+1 (global)
     sts_quad<kSlots>(tn + T::tC, c0.C);  // old C(k+1), D(k+1): z+ / x,y neighbours now,
@@ -355,13 +373,13 @@ __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long it
     // upper half-step: A(k+1) from C(k+1), C(k), D(k+1); B(k) from D(k+1), D(k), C(k)
     const Quad oC0 = lds_quad<kSlots>(tk + T::tC), oC1 = lds_quad<kSlots>(tk + T::tC + TW);  // old C(k) of the two cells
     const Quad nA0 = update(IA{}, 0, c0.A, c0.D, tn + T::tD, lds_value<kSlots>(tn + T::tD + YM, 1), qlane(c1.D, 0), c0.C, oC0, Zn,
-                            zq0, on0, ok0, nullptr, &sLk[pk][0]);
+                            zq0, on0, rn0, nullptr, &sLk[pk][0]);
     const Quad nA1 = update(IA{}, 1, c1.A, c1.D, tn + T::tD + TW, qlane(c0.D, 1), lds_value<kSlots>(tn + T::tD + YP, 0), c1.C, oC1,
-                            Zn, zq0, on1, ok1, nullptr, &sLk[pk][0]);
+                            Zn, zq0, on1, rn1, nullptr, &sLk[pk][0]);
     const Quad nB0 = update(IB{}, 0, c0.B, oC0, tk + T::tC, lds_value<kSlots>(tk + T::tC + YM, 1), qlane(oC1, 0), c0.D,
-                            lds_quad<kSlots>(tk + T::tD), Zk + 1, zq1, ok0, ok0, nullptr, &sLk[pk][1]);
+                            lds_quad<kSlots>(tk + T::tD), Zk + 1, zq1, ok0, rk0, nullptr, &sLk[pk][1]);
     const Quad nB1 = update(IB{}, 1, c1.B, oC1, tk + T::tC + TW, qlane(oC0, 1), lds_value<kSlots>(tk + T::tC + YP, 0), c1.D,
-                            lds_quad<kSlots>(tk + T::tD + TW), Zk + 1, zq1, ok1, ok1, nullptr, &sLk[pk][1]);
+                            lds_quad<kSlots>(tk + T::tD + TW), Zk + 1, zq1, ok1, rk1, nullptr, &sLk[pk][1]);
     sts_quad<kSlots>(tk + T::tB, nB0);
     sts_quad<kSlots>(tn + T::tA, nA0);
     sts_quad<kSlots>(tk + T::tB + TW, nB1);
@@ -381,10 +399,10 @@ __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long it
                        // the halo cells too, to interleave the two cells, was slower)
           float lc = 0.0f;
           const Quad nC = update(IC{}, 0, oC0, nB0, tk + T::tB, lds_value<kSlots>(tk + T::tB + YM, 1), qlane(nB1, 0), nA0, oA0,
-                                 Zk + 1, zq1, ok0, ok0, Sp, &sLk[pk][2]);
+                                 Zk + 1, zq1, ok0, rk0, Sp, &sLk[pk][2]);
           if (kE) lc = cross(nC, S, lc);
           const Quad nD = update(ID{}, 0, lds_quad<kSlots>(tk + T::tD), oA0, tk + T::tA, lds_value<kSlots>(tk + T::tA + YM, 1),
-                                 qlane(oA1, 0), nB0, lds_quad<kSlots>(tn + T::tB), Zk, zq2, ok0, ok0, Sp, &sLk[pk][3]);
+                                 qlane(oA1, 0), nB0, lds_quad<kSlots>(tn + T::tB), Zk, zq2, ok0, rk0, Sp, &sLk[pk][3]);
           if (core0) {
             if (kE) {  // this level's few terms in FP32, the running sums in FP64 (shared memory)
               e_acc[1] += cross(nD, S, lc);
@@ -398,10 +416,10 @@ __device__ __forceinline__ void fused3d_item(const FusedArgs<P>& a, long long it
         if (!th.h1) {  // cell 1 (warp-uniform)
           float lc = 0.0f;
           const Quad nC = update(IC{}, 1, oC1, nB1, tk + T::tB + TW, qlane(nB0, 1), lds_value<kSlots>(tk + T::tB + YP, 0), nA1,
-                                 oA1, Zk + 1, zq1, ok1, ok1, Sp, &sLk[pk][2]);
+                                 oA1, Zk + 1, zq1, ok1, rk1, Sp, &sLk[pk][2]);
           if (kE) lc = cross(nC, S, lc);
           const Quad nD = update(ID{}, 1, lds_quad<kSlots>(tk + T::tD + TW), oA1, tk + T::tA + TW, qlane(oA0, 1),
-                                 lds_value<kSlots>(tk + T::tA + YP, 0), nB1, lds_quad<kSlots>(tn + T::tB + TW), Zk, zq2, ok1, ok1, Sp,
+                                 lds_value<kSlots>(tk + T::tA + YP, 0), nB1, lds_quad<kSlots>(tn + T::tB + TW), Zk, zq2, ok1, rk1, Sp,
                                  &sLk[pk][3]);
           if (core1) {
             if (kE) {

@@ -159,9 +159,11 @@ void launch_link_table(void* tab, int n, const FieldDesc& f, int dims, int axis,
 
 // coefficient table of a time-independent potential (COEF_TABLE): every
 // plane of the state layout (pstride), b = 1/(1 + i dt (beta m + V)/2) as
-// {re hi, im hi, re lo, im lo}, or (quads) as the quad records of quad.cuh
+// {re hi, im hi, re lo, im lo}, or (quads) as the quad records of quad.cuh.
+// rep (device, or null): N are the classes per axis and rep, axis after axis,
+// one cell coordinate of each
 void launch_coef_table(float4* tab, const FieldDesc& f, int dims, const int N[3], long long pstride, int quads,
-                       cudaStream_t s);
+                       const int* rep, cudaStream_t s);
 
 // the FP64 kernels' table: alpha and gamma of every value, tab[plane * pstride + cell]
 void launch_coef64_table(F64::Coef* tab, const FieldDesc& f, int dims, const int N[3], long long pstride,

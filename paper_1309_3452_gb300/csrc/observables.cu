@@ -329,12 +329,13 @@ __global__ void link_table_kernel(typename PlaneLinkOf<P>::type* tab, int n, con
 // potentials only); stored as {re hi, im hi, re lo, im lo}
 template <int DIMS>
 __global__ void coef_table_kernel(float4* __restrict__ tab, const FieldDesc f, int N0, int N1, int N2,
-                                  long long pstride, int quads) {
+                                  long long pstride, int quads, const int* __restrict__ rep) {
   const int plane = blockIdx.y;
   const long long ncell = (long long)N0 * N1 * N2;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
        c += (long long)gridDim.x * blockDim.x) {
-    const long long x = c % N0, y = (c / N0) % N1, z = c / ((long long)N0 * N1);
+    long long x = c % N0, y = (c / N0) % N1, z = c / ((long long)N0 * N1);
+    if (rep) x = rep[x], y = rep[N0 + y], z = rep[N0 + N1 + z];
     const long long X = 2 * x + plane_off<DIMS>(plane, 0), Y = 2 * y + plane_off<DIMS>(plane, 1),
                     Z = DIMS == 3 ? 2 * z + plane_off<DIMS>(plane, 2) : 0;
     const double V = potential_at(f, DIMS, X, Y, Z, c, pstride, plane, 0.0);
@@ -645,15 +646,15 @@ template void launch_link_table<F32>(void*, int, const FieldDesc&, int, int, int
                                      cudaStream_t);
 
 void launch_coef_table(float4* tab, const FieldDesc& f, int dims, const int N[3], long long pstride, int quads,
-                       cudaStream_t s) {
+                       const int* rep, cudaStream_t s) {
   const long long ncell = (long long)N[0] * N[1] * (dims == 3 ? N[2] : 1);
   long long bx = (ncell + 255) / 256;
   if (bx > 152 * 16) bx = 152 * 16;
   const dim3 grid((unsigned)bx, dims == 3 ? 8 : 4);
   if (dims == 3)
-    coef_table_kernel<3><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], N[2], pstride, quads);
+    coef_table_kernel<3><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], N[2], pstride, quads, rep);
   else
-    coef_table_kernel<2><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], 1, pstride, quads);
+    coef_table_kernel<2><<<grid, 256, 0, s>>>(tab, f, N[0], N[1], 1, pstride, quads, rep);
 }
 
 void launch_coef64_table(F64::Coef* tab, const FieldDesc& f, int dims, const int N[3], long long pstride,

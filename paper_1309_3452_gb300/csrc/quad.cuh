@@ -181,19 +181,19 @@ __device__ __forceinline__ Quad apply_table_quad(float4 bh, float4 bl, float rxh
 __device__ __forceinline__ float4 lanes_of(float4 r0, float4 r1) { return make_float4(r0.x, r1.y, r0.z, r1.w); }
 
 // The update of both values of component comp (planes 2 comp and 2 comp + 1).
-// up, dn: the neighbours at +-dx_a/2 of each lane's value; H0, H1 and site0,
-// site1: each lane's half-lattice point and cell.  bpre: the coefficients of
+// up, dn: the neighbours at +-dx_a/2 of each lane's value; H0, H1, site0, site1
+// and class0, class1: each lane's half-lattice point, cell and class (COEF_TABLE).  bpre: the coefficients of
 // the pair where the caller forms them (COEF_SOFTCORE, COEF_SOFTCORR); lk: the
 // staged link factor of LINK_PLANE_ZX; lanes: COEF_LANES; w0, w1: the lanes'
 // factors (c_hi, c_lo, s_hi, s_lo) of LINK_PLANE.
-// kOneCell: site0 == site1.  kIso: r_x = r_y = r_z (a template parameter: a
+// kOneCell: site0 == site1, class0 == class1.  kIso: r_x = r_y = r_z (a template parameter: a
 // test here, uniform as it is, would end the compiler's basic block at every
 // component and keep it from overlapping the chains of the others).
 template <int DIMS, int COEF, int LINK, bool kOneCell, bool kIso>
 __device__ __forceinline__ Quad quad_update(const HalfFields<F32>& h, const FieldDesc& f, bool iso,
                                             const F32::Ratio& ry, const F32::Ratio& rz, int comp, const Quad& F,
                                             const Quad (&up)[3], const Quad (&dn)[3], const int (&H0)[3],
-                                            const int (&H1)[3], long long site0, long long site1, long long pstride,
+                                            const int (&H1)[3], long long site0, long long site1, long long class0, long long class1, long long pstride,
                                             Quad* S_out, const SoftB2* bpre, const PlaneLink32* lk,
                                             const int (&N)[3], const float4* lanes = nullptr,
                                             const float4* w0 = nullptr, const float4* w1 = nullptr) {
@@ -272,11 +272,11 @@ __device__ __forceinline__ Quad quad_update(const HalfFields<F32>& h, const Fiel
       }
       return r;
     } else if constexpr (COEF == COEF_TABLE) {
-      const float4* t = h.bq + 2 * (long long)comp * h.q_ps;
-      float4 bh = __ldg(t + 2 * site0), bl = __ldg(t + 2 * site0 + 1);
+      const float4* t = h.bq + 2 * (long long)comp * h.b_ps;
+      float4 bh = __ldg(t + 2 * class0), bl = __ldg(t + 2 * class0 + 1);
       if (!kOneCell) {
-        bh = lanes_of(bh, __ldg(t + 2 * site1));
-        bl = lanes_of(bl, __ldg(t + 2 * site1 + 1));
+        bh = lanes_of(bh, __ldg(t + 2 * class1));
+        bl = lanes_of(bl, __ldg(t + 2 * class1 + 1));
       }
       return apply_table_quad(bh, bl, h.rx_hi, h.rx_lo, F, S);
     } else if constexpr (COEF == COEF_SOFTCORE || COEF == COEF_SOFTCORR) {
