@@ -1305,13 +1305,16 @@ static dirac_status batch_group(dirac_sim* const* g, int n, long nsteps) {
   }
   const long launches = passes.launches();
   std::vector<int> chunks(kBatchModes * n, 0);
-  for (int i = 0; i < n; ++i) {
-    dirac_sim* s = g[i];
-    for (int m = 0; m < kBatchModes; ++m) {
-      if (!passes.count[m]) continue;
-      const int planned = m ? s->chunk2 : s->chunk1;
-      chunks[kBatchModes * i + m] = planned > 0 ? planned : fused_chunk(s->dims, s->N, m + 1);
+  std::vector<const int*> extents(n);
+  std::vector<int> chunk(n);
+  for (int m = 0; m < kBatchModes; ++m) {
+    if (!passes.count[m]) continue;
+    for (int i = 0; i < n; ++i) {
+      extents[i] = g[i]->N;
+      chunk[i] = m ? g[i]->chunk2 : g[i]->chunk1;  // planned, or 0
     }
+    fused_batch_chunks(s0->dims, extents.data(), n, m + 1, chunk.data());
+    for (int i = 0; i < n; ++i) chunks[kBatchModes * i + m] = chunk[i];
   }
   const bool use_graph = launches <= kBatchGraphMaxLaunches && std::getenv("DIRAC_NO_GRAPHS") == nullptr;
 

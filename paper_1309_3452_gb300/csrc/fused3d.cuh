@@ -7,9 +7,10 @@
 // (3+1)D: a block of 480 threads covers a 34 x 28 tile of cells in (x, y), or
 // 512 threads a 34 x 30 one, and marches along z; every thread updates two
 // cells stacked in y (rows ly, ly + 1), so the y neighbour inside the pair
-// comes from registers.  Columns 0, 33 and the first and last row are a one-cell halo: they load and compute the upper
-// half-step like every other cell, so the new upper values the interior needs from outside the tile exist in shared memory, but they store
-// nothing.  Per z level k the block
+// comes from registers.  Columns 0, 33 and the first and last row are a one-cell
+// halo: they load and compute the upper half-step like every other cell, so the
+// new upper values the interior needs from outside the tile exist in shared
+// memory, but they store nothing.  Per z level k the block
 //   1. holds the old A(k+1), C(k+1), D(k+1) and B(k) (B, C sit at z+1/2) in
 //      registers, loaded while level k-1 was computed, publishes C(k+1) and
 //      D(k+1) in shared memory and starts the loads of level k+1,
@@ -28,6 +29,16 @@
 // neighbouring tiles at the same levels at the same time and the overlapping
 // halo loads hit L2.  The chunk length balances full rounds against the one
 // restart level of each item.
+//
+// Bound: the FP32 pipe and the latency of a level's two barriers with 15 or 16
+// warps on an SM (a free 128^3 step takes 54 us, its 128 bytes per cell 40 at the
+// copy rate; a soft core's coefficients alone keep the FP32 pipe busy for a
+// third of the laser's time).  Tiles of 34 x 28 and 34 x 30 cells are the largest whose
+// four components fit the registers of one block per SM: smaller ones spend more
+// on halo cells (14 rows: 6114 us per 512^3 laser step against 3931).  us per
+// step, with (re, im) lanes per value / now: 128^3 free 59.6 / 54.4, 203 x 149 x
+// 91 Klein step anisotropic 102 / 82.8, 512^3 laser 4879 / 3945, 160^3 layers
+// 227 / 141, 128^3 static links 670 / 395.
 //
 // Cells outside the grid (ragged last tiles) are wrapped periodically, so
 // they compute correct duplicates and only the owning interior thread stores.
@@ -514,8 +525,8 @@ int workers3d() {
 // their rows, halo and ragged last tile included); 15 pairs at equal rows are 5 %
 // faster with a soft core (its arithmetic fills the four schedulers evenly; 512^3 laser
 // 3931 us per step against 4084 with 14 pairs, 570 rows against 560) and even
-// otherwise (160^3 layers 189 us per step with 15 pairs, 180 rows, against 206
-// with 14, 196 rows; 128^3 free 57.7 against 54.2, 150 rows against 140).
+// otherwise (160^3 layers with a coefficient record per cell 189 us per step with
+// 15 pairs, 180 rows, against 206 with 14, 196 rows; 128^3 free 57.7 against 54.2, 150 rows against 140).
 template <int COEF>
 bool taller_tile(const int N[3]) {
   const long long r14 = (N[1] + Tile3<14>::CY - 1) / Tile3<14>::CY * Tile3<14>::TH;

@@ -106,6 +106,9 @@ struct BatchArgs {
 // (a FusedArgs chunk of 0 makes the launchers take fused_chunk's rule), with
 // `steps` time steps per pass (1; (2+1)D: 1 or 2)
 int fused_chunk(int dims, const int N[3], int steps);
+// the same for n grids in one batched launch (N[i] the extents): every chunk[i]
+// that is 0 is set
+void fused_batch_chunks(int dims, const int* const* N, int n, int steps, int* chunk);
 // chunk lengths worth timing, best first by the planner's model; returns the count
 int fused_candidates(int dims, const int N[3], int steps, int* out, int max);
 long long fused_items(int dims, const int N[3], int steps, int chunk);

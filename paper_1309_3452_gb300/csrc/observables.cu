@@ -503,6 +503,8 @@ __global__ void convert_out_kernel(const float2* __restrict__ src, double2* __re
     dst[i] = make_double2(src[i].x, src[i].y);
 }
 
+// Bound: HBM (32 B in and 16 B out per cell and component, or back): both planes
+// of a component in one pass, so that the quads are written whole.
 // two canonical planes <-> one component's quads; lane < 0: both planes, else
 // the one plane of that sublattice (src0 / dst0)
 __global__ void convert_in_quads_kernel(const double2* __restrict__ src0, const double2* __restrict__ src1,

@@ -4,6 +4,13 @@
 // the other parity (Eqs. ss1-ss4: A,B from C,D at t; C,D from the new A,B).
 // This is the plain reference path (and the FP64 validation path); the fused
 // kernels compute the same values with the same per-value arithmetic.
+//
+// Bound, FP64: the FP64 pipe (0.5e12 instructions per second on the whole GPU;
+// 144 per free (3+1)D cell and step are 246 us at 96^3, measured 249), so what
+// counts is that nothing but the update runs on it: potentials and link factors
+// come from tables.  us per step, before and now: 64^3 soft core in a plane wave
+// 1388 / 131 (per-site square roots, divisions and sines before), 96^3 free
+// 254 / 249, 64^2 free 5.5 / 5.0 (two launches).
 #include "fused_common.cuh"
 
 namespace dirac {
