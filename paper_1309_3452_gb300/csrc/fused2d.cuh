@@ -11,11 +11,11 @@
 // arithmetic.  Every step loses one lane and one row per side, so the arithmetic
 // grows by 32 / (32 - 2 kT) and the restart of an item by kT rows.
 //
-// Bound: instruction issue (about 145 thread instructions per cell and step,
-// 64 % of the issue slots; HBM at half its rate).  us per step with one warp row
-// of (re, im) lanes per value / with quads and stages waiting for one another /
+// Bound: instruction issue (147 thread instructions per cell and step, 66 % of
+// the issue slots, FP32 pipe 50 %, ALU 41 %; HBM at 68 % of its peak).  us per
+// step with one warp row of (re, im) lanes per value / with quads and stages waiting for one another /
 // now: 4096^2 Klein step 138 / 131 / 95, 1000^2 moving plane wave 35.0 / 26.8 /
-// 16.6 (one step per pass before), 300 x 260 constant A 16.8 / 13.7 / 3.2 (blocks of
+// 13.5 (one step per pass before), 300 x 260 constant A 16.8 / 13.7 / 3.1 (blocks of
 // eight warps and chunks of 32 rows left most SMs idle).  Four steps per pass
 // were measured too: 4096^2 103 (spills or 8 warps per SM), 300 x 260 2.95.
 #pragma once

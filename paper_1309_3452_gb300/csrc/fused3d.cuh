@@ -30,13 +30,14 @@
 // halo loads hit L2.  The chunk length balances full rounds against the one
 // restart level of each item.
 //
-// Bound: the FP32 pipe and the latency of a level's two barriers with 15 or 16
-// warps on an SM (a free 128^3 step takes 54 us, its 128 bytes per cell 40 at the
-// copy rate; a soft core's coefficients alone keep the FP32 pipe busy for a
-// third of the laser's time).  Tiles of 34 x 28 and 34 x 30 cells are the largest whose
-// four components fit the registers of one block per SM: smaller ones spend more
-// on halo cells (14 rows: 6114 us per 512^3 laser step against 3931).  us per
-// step, with (re, im) lanes per value / now: 128^3 free 59.6 / 54.4, 203 x 149 x
+// Bound: without fields the shared-memory queue and the two barriers of a level
+// (2.6 and 1.6 of the stalled warps per issue at 128^3, the FP32 pipe 31 % busy;
+// 54 us per step, its 128 bytes per cell take 40 at the copy rate); with a soft
+// core and a plane wave the FP32 pipe (52 % busy over the kernel, stalled on it
+// in the long chains) and the barriers.  Tiles of 34 x 28 and 34 x 30 cells are
+// the largest that one block per SM can hold two cells per thread of: smaller
+// ones spend more on halo cells (14 rows: 6114 us per 512^3 laser step against
+// 3931).  us per step, with (re, im) lanes per value / now: 128^3 free 59.6 / 54.4, 203 x 149 x
 // 91 Klein step anisotropic 102 / 82.8, 512^3 laser 4879 / 3945, 160^3 layers
 // 227 / 141, 128^3 static links 670 / 395.
 //
