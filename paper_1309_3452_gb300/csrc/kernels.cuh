@@ -13,7 +13,7 @@ namespace dirac {
 // its writes are visible.  Every kernel launched this way calls depends() before
 // it touches memory, so the order of all work is that of plain launches; what
 // is saved is the launch latency between short kernels.
-// us per step, before and after: 96^3 FP64 254 / 249, 64^3 laser FP64 142 / 136,
+// us per step, before and after: 96^3 FP64 254 / 249, 64^2 FP64 5.5 / 5.0,
 // 203x149x91 84.5 / 82.8, 300 x 260 3.16 / 3.09; long kernels unchanged.
 __device__ __forceinline__ void depends() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
