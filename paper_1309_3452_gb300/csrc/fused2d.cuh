@@ -256,6 +256,9 @@ __device__ __forceinline__ void march2d(const FusedArgs<P>& a, float4* ring, int
     }
   }
   cp_async_wait<0>();  // nothing of this item lands in the next one's slots
+  // every lane has read its last factors before a few lanes write the next item's
+  // (the rows in the ring are each lane's own)
+  if (LINK == LINK_PLANE) __syncwarp();
 }
 
 template <class P, int COEF, int LINK, int kT, bool kIso>

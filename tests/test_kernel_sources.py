@@ -1,0 +1,31 @@
+"""Orderings the kernels rely on, read in their sources: a missing one is a race
+that a run may or may not show."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1309_3452_gb300", "csrc")
+
+
+def source(name):
+    """The file's code without comments."""
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"/\*.*?\*/", "", re.sub(r"//[^\n]*", "", f.read()), flags=re.S)
+
+
+def body(text, head):
+    """The braces that follow the first `head`."""
+    i = text.index("{", text.index(head))
+    depth = 0
+    for j in range(i, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[j], 0)
+        if depth == 0:
+            return text[i + 1:j]
+    raise ValueError(head)
+
+
+def test_strip_items_end_with_a_warp_barrier():
+    """A wave's factors are written by a few lanes and read by all: between the last read of one item
+    and the first write of the warp's next item all lanes meet."""
+    march = body(source("fused2d.cuh"), "void march2d(")
+    tail = march[march.rindex("cp_async_wait<0>()"):]
+    assert re.search(r"if \(LINK == LINK_PLANE\) __syncwarp\(\);", tail)
