@@ -181,10 +181,10 @@ __device__ __forceinline__ void march2d(const FusedArgs<P>& a, float4* ring, int
   };
   if (LINK == LINK_PLANE) {
     if (wave_y) {
-      if (lane < 4 * kT) wave[(k0 & (kWaveRows - 1)) * 8 + lane] = __ldg(wave_entry(lane, 2 * gy(k0)));
+      if (lane < 4 * kT) wave[(k0 & (kWaveRows - 1)) * 8 + lane] = *wave_entry(lane, 2 * gy(k0));
     } else {
 #pragma unroll
-      for (int e = 0; e < 4 * kT; ++e) wave[e * 32 + lane] = __ldg(wave_entry(e, hx));
+      for (int e = 0; e < 4 * kT; ++e) wave[e * 32 + lane] = *wave_entry(e, hx);  // (ordinary loads, as ldq)
     }
   }
 #pragma unroll

@@ -26,7 +26,11 @@ struct Quad {
 };
 __device__ __forceinline__ Quad quad(float4 v) { return Quad{make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
 __device__ __forceinline__ float4 pack4(const Quad& q) { return make_float4(q.re.x, q.re.y, q.im.x, q.im.y); }
-__device__ __forceinline__ Quad ldq(const float4* p) { return quad(__ldg(p)); }
+// A record of the evolving state: an ordinary load.  The read-only path (__ldg) may
+// be used for what no kernel writes while this one is resident, and a step is
+// resident (waiting in depends()) while the step before writes the state and the
+// launch before that a wave's link table.
+__device__ __forceinline__ Quad ldq(const float4* p) { return quad(*p); }
 __device__ __forceinline__ float2 qlane(const Quad& q, int l) {
   return l ? make_float2(q.re.y, q.im.y) : make_float2(q.re.x, q.im.x);
 }

@@ -1,4 +1,4 @@
-"""Work items that follow one another on a warp, bit for bit
+"""Launches, and a warp's work items, that follow one another without a gap, bit for bit
 against the plain half-step kernels (which form every value by the same
 operations)."""
 import math
@@ -43,3 +43,19 @@ def test_many_strip_items_per_warp_with_a_moving_wave(D, axis, step):
     psi = W.random_state(prob, 17)
     out = run(D, prob, psi, 67, plan=dict(chunk=1, two_step=1, chunk2=1))
     assert np.array_equal(out, run(D, prob, psi, 67, flags=D.FLAG_REFERENCE_KERNELS))
+
+
+@pytest.mark.parametrize("graphs", [True, False])
+@pytest.mark.parametrize("dims,N", [(2, (700, 300, 1)), (3, (96, 84, 40)), (3, (40, 36, 160))])
+@pytest.mark.parametrize("field", ["free", "wave", "softcore"])
+def test_hundreds_of_launches_over_a_state_in_cache(D, monkeypatch, graphs, dims, N, field):
+    """A step starts while the blocks of the one before still write what it reads."""
+    if not graphs:
+        monkeypatch.setenv("DIRAC_NO_GRAPHS", "1")
+    k = [0.0, 0.0, 0.0]
+    k[dims - 1] = 2 * math.pi / N[dims - 1]
+    f = {"free": {}, "wave": dict(q=1.0, Apw_amp=0.5, Apw_k=tuple(k), Apw_omega=0.3, Apw_pol=0),
+         "softcore": dict(sc_Z=1.0, sc_a=1.0, sc_center=tuple(n / 2 for n in N))}[field]
+    prob = W.Problem(dims, N, (1.0, 1.0, 1.0), 0.9 * W.stability_limit(dims), 0.4, W.Fields(**f))
+    psi = W.random_state(prob, 23)
+    assert np.array_equal(run(D, prob, psi, 401), run(D, prob, psi, 401, flags=D.FLAG_REFERENCE_KERNELS))

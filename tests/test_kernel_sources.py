@@ -3,6 +3,8 @@ that a run may or may not show."""
 import os
 import re
 
+import pytest
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1309_3452_gb300", "csrc")
 
 
@@ -29,3 +31,19 @@ def test_strip_items_end_with_a_warp_barrier():
     march = body(source("fused2d.cuh"), "void march2d(")
     tail = march[march.rindex("cp_async_wait<0>()"):]
     assert re.search(r"if \(LINK == LINK_PLANE\) __syncwarp\(\);", tail)
+
+
+# what a fused step may read through the read-only path: tables made with the simulation, and the
+# argument tables of a batched call, uploaded before its first launch
+FIXED = ("sc_sq", "b_map", "class_z", "sc_corr", "t + 2 *", "first + mid", "s + i")
+
+
+@pytest.mark.parametrize("name", ["quad.cuh", "fused2d.cuh", "fused3d.cuh", "fused_common.cuh"])
+def test_evolving_data_is_read_by_ordinary_loads(name):
+    """A dependent launch is resident while the one before it writes the state and a wave's factors."""
+    text = source(name)
+    for m in re.finditer(r"__ldg\(", text):
+        arg = text[m.end():m.end() + 60]
+        assert any(f in arg for f in FIXED), arg
+    # "t" in quad.cuh is the static link table or the coefficient table
+    assert set(re.findall(r"const float4\* t = ([\w.]+)", text)) <= {"h.lq", "h.bq"}
