@@ -104,6 +104,14 @@ static dirac_status cuda_fail(dirac_sim* s, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail((sim), e_, #call); \
   } while (0)
 
+// A host table to the device on the simulation's stream (one that need not be
+// ordered after the legacy stream, where a plain copy of pageable memory may still
+// be under way when it returns); the host memory may go when this returns
+static cudaError_t upload(const dirac_sim* s, void* dst, const void* src, size_t bytes) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s->stream);
+  return e == cudaSuccess ? cudaStreamSynchronize(s->stream) : e;
+}
+
 static long long round_up(long long v, long long m) { return (v + m - 1) / m * m; }
 
 static long long cells_of(int dims, const int N[3]) {
@@ -708,9 +716,8 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
     softcore_tables(s, sq);
     if ((e = cudaMalloc(&s->sc_sq, sq.size() * sizeof(float2))) != cudaSuccess)
       return cleanup_fail(cuda_fail(s, e, "cudaMalloc(soft-core tables)"));
-    // synchronous: the host vector goes out of scope
-    if ((e = cudaMemcpy(s->sc_sq, sq.data(), sq.size() * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess)
-      return cleanup_fail(cuda_fail(s, e, "cudaMemcpy(soft-core tables)"));
+    if ((e = upload(s, s->sc_sq, sq.data(), sq.size() * sizeof(float2))) != cudaSuccess)
+      return cleanup_fail(cuda_fail(s, e, "upload(soft-core tables)"));
   }
   if (s->coef_mode == COEF_SOFTCORR) {
     // the correction records, built on the device; if one does not fit its
@@ -775,9 +782,8 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
       if (shared) s->b_ps = (long long)classes[0] * classes[1] * classes[2];
       if ((e = cudaMalloc(&s->b_map, map.size() * sizeof(unsigned))) != cudaSuccess)
         return cleanup_fail(cuda_fail(s, e, "cudaMalloc(coefficient classes)"));
-      // synchronous: the host vector goes out of scope
-      if ((e = cudaMemcpy(s->b_map, map.data(), map.size() * sizeof(unsigned), cudaMemcpyHostToDevice)) != cudaSuccess)
-        return cleanup_fail(cuda_fail(s, e, "cudaMemcpy(coefficient classes)"));
+      if ((e = upload(s, s->b_map, map.data(), map.size() * sizeof(unsigned))) != cudaSuccess)
+        return cleanup_fail(cuda_fail(s, e, "upload(coefficient classes)"));
       if (shared) rep = reinterpret_cast<const int*>(s->b_map) + s->N[0] + s->N[1] + s->N[2];
     }
     if ((e = cudaMalloc(&s->b_tab, (size_t)s->np * s->b_ps * sizeof(float4))) != cudaSuccess)

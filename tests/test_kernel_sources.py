@@ -47,3 +47,9 @@ def test_evolving_data_is_read_by_ordinary_loads(name):
         assert any(f in arg for f in FIXED), arg
     # "t" in quad.cuh is the static link table or the coefficient table
     assert set(re.findall(r"const float4\* t = ([\w.]+)", text)) <= {"h.lq", "h.bq"}
+
+
+def test_no_copies_on_the_legacy_stream():
+    """Kernels on a non-blocking stream are not ordered after what goes through the legacy one."""
+    for name in sorted(os.listdir(CSRC)):
+        assert not re.search(r"\bcuda(Memcpy|Memset)\(", source(name)), name
