@@ -45,18 +45,21 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NS], double* out)
 
 // Running sums of a thread: FP64 for FP64 states.  For FP32 states the FP64
 // pipe (1.6 lanes per clock and SM) would be the limit, so a cell's terms are
-// added to an unevaluated sum hi + lo of two floats (TwoSum: the rounding error
-// of every addition is kept, relative error of the sum below 2^-44), which
-// goes to FP64 every kFlush cells: over the ~10^3 cells of a thread no less
-// exact than FP64 additions one by one.
+// added to an unevaluated sum h + m + l of three floats: the rounding error of
+// h goes to m, that of m to l (TwoSum, both exact), so only l rounds, by 2^-24 of
+// itself, at most 2^-64 of the largest partial sum over the kFlush cells after which
+// the three go to FP64.  FP64 additions one by one round by 2^-53 of the sum each.
 constexpr int kFlush = 16;
 struct Sum32 {
-  float h, l;
-  __device__ __forceinline__ void add(float v) {
-    const float s = __fadd_rn(h, v), b = __fsub_rn(s, h);
-    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(v, b)));
-    h = s;
+  float h, m, l;
+  // s becomes s + v, the result is what the rounding left out
+  static __device__ __forceinline__ float two_sum(float& s, float v) {
+    const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b));
+    s = t;
+    return e;
   }
+  __device__ __forceinline__ void add(float v) { l = __fadd_rn(l, two_sum(m, two_sum(h, v))); }
   // f v with f = fh + fl: the product's error by FMA
   __device__ __forceinline__ void add_product(float fh, float fl, float v) {
     const float p = __fmul_rn(fh, v);
@@ -64,8 +67,8 @@ struct Sum32 {
     add(p);
   }
   __device__ __forceinline__ void flush(double& acc) {
-    acc += (double)h + (double)l;
-    h = l = 0.0f;
+    acc += (double)h + ((double)m + (double)l);
+    h = m = l = 0.0f;
   }
 };
 struct Sum64 {
