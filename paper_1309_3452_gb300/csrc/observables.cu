@@ -2,6 +2,8 @@
 // conserved functional (Lemma of Sect. 2, Eq. EPM, in its "lower" form; see
 // dirac.h) and the partial density used for the Klein-step transmission; and
 // the tables and layout conversions that a simulation is set up with.
+#include <cfloat>
+
 #include "kernels.cuh"
 #include "fused_common.cuh"
 
@@ -81,6 +83,34 @@ struct Sum64 {
 };
 template <class P> struct SumOf { using type = Sum64; };
 template <> struct SumOf<F32> { using type = Sum32; };
+
+// L up - conj(M) dn of FP32 values rounded once: each part is a sum of four
+// products formed as by Dot2 (Ogita, Rump, Oishi, SIAM J. Sci. Comput. 26, 2005),
+// the products of the factors' lo parts among the corrections, so that what is
+// left out is about 2^-47 of the neighbours.  (A product rounded to FP32 before the
+// difference is taken leaves out 2^-24 of them, however small the difference;
+// FP64 arithmetic would put 20 operations per link on the narrow FP64 pipe.)
+struct Dot32 {
+  float s, e;
+  __device__ __forceinline__ void add(float f_hi, float f_lo, float v) {
+    const float p = __fmul_rn(f_hi, v), pe = __fmaf_rn(f_hi, v, -p);
+    e = __fadd_rn(e, __fmaf_rn(f_lo, v, __fadd_rn(pe, Sum32::two_sum(s, p))));
+  }
+  // (an infinite product leaves no corrections)
+  __device__ __forceinline__ float value() const { return fabsf(e) <= FLT_MAX ? __fadd_rn(s, e) : s; }
+};
+__device__ __forceinline__ float2 rotated_diff(const F32::Link& L, float2 up, const F32::Link& M, float2 dn) {
+  Dot32 re{}, im{};
+  re.add(L.hi.x, L.lo.x, up.x);
+  re.add(-L.hi.y, -L.lo.y, up.y);
+  re.add(-M.hi.x, -M.lo.x, dn.x);
+  re.add(-M.hi.y, -M.lo.y, dn.y);
+  im.add(L.hi.x, L.lo.x, up.y);
+  im.add(L.hi.y, L.lo.y, up.x);
+  im.add(-M.hi.x, -M.lo.x, dn.y);
+  im.add(M.hi.y, M.lo.y, dn.x);
+  return make_float2(re.value(), im.value());
+}
 
 // Both values of a component in one cell (two planes, or one quad).
 template <class P>
@@ -224,14 +254,16 @@ __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
               up = link_mul(up_link<P>(t + (plane * a.pstride + cell)), up);
               dn = link_mulc(up_link<P>(t + (partner<DIMS>(plane, ax) * a.pstride + below)), dn);
             }
+            re = up.x - dn.x;
+            im = up.y - dn.y;
             if constexpr (kLink == LINK_TABLE && kQuads) {
               const float4* t = a.lq + 2 * ((long long)(2 * ax * nc + c) * a.pstride + cell);
               const float4 u = quad_lane(t, l), d = quad_lane(t + 2 * nc * a.pstride, l);
-              up = link_mul(F32::Link{make_float2(u.x, u.y), make_float2(u.z, u.w)}, up);
-              dn = link_mulc(F32::Link{make_float2(d.x, d.y), make_float2(d.z, d.w)}, dn);
+              const C w = rotated_diff(F32::Link{make_float2(u.x, u.y), make_float2(u.z, u.w)}, up,
+                                       F32::Link{make_float2(d.x, d.y), make_float2(d.z, d.w)}, dn);
+              re = w.x;
+              im = w.y;
             }
-            re = up.x - dn.x;
-            im = up.y - dn.y;
           }
           const R sre = ax == 1 ? (p ? -im : im) : (ax == 2 && p ? -re : re);
           const R sim = ax == 1 ? (p ? re : -re) : (ax == 2 && p ? -im : im);
