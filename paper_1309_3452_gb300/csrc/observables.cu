@@ -62,12 +62,6 @@ struct Sum32 {
     return e;
   }
   __device__ __forceinline__ void add(float v) { l = __fadd_rn(l, two_sum(m, two_sum(h, v))); }
-  // f v with f = fh + fl: the product's error by FMA
-  __device__ __forceinline__ void add_product(float fh, float fl, float v) {
-    const float p = __fmul_rn(fh, v);
-    l = __fmaf_rn(fl, v, __fadd_rn(l, __fmaf_rn(fh, v, -p)));
-    add(p);
-  }
   __device__ __forceinline__ void flush(double& acc) {
     acc += (double)h + ((double)m + (double)l);
     h = m = l = 0.0f;
@@ -92,6 +86,10 @@ template <> struct SumOf<F32> { using type = Sum32; };
 // FP64 arithmetic would put 20 operations per link on the narrow FP64 pipe.)
 struct Dot32 {
   float s, e;
+  __device__ __forceinline__ Dot32(float f_hi, float f_lo, float v) {
+    s = __fmul_rn(f_hi, v);
+    e = __fmaf_rn(f_lo, v, __fmaf_rn(f_hi, v, -s));
+  }
   __device__ __forceinline__ void add(float f_hi, float f_lo, float v) {
     const float p = __fmul_rn(f_hi, v), pe = __fmaf_rn(f_hi, v, -p);
     e = __fadd_rn(e, __fmaf_rn(f_lo, v, __fadd_rn(pe, Sum32::two_sum(s, p))));
@@ -100,12 +98,10 @@ struct Dot32 {
   __device__ __forceinline__ float value() const { return fabsf(e) <= FLT_MAX ? __fadd_rn(s, e) : s; }
 };
 __device__ __forceinline__ float2 rotated_diff(const F32::Link& L, float2 up, const F32::Link& M, float2 dn) {
-  Dot32 re{}, im{};
-  re.add(L.hi.x, L.lo.x, up.x);
+  Dot32 re(L.hi.x, L.lo.x, up.x), im(L.hi.x, L.lo.x, up.y);
   re.add(-L.hi.y, -L.lo.y, up.y);
   re.add(-M.hi.x, -M.lo.x, dn.x);
   re.add(-M.hi.y, -M.lo.y, dn.y);
-  im.add(L.hi.x, L.lo.x, up.y);
   im.add(L.hi.y, L.lo.y, up.x);
   im.add(-M.hi.x, -M.lo.x, dn.y);
   im.add(M.hi.y, M.lo.y, dn.x);
@@ -132,9 +128,7 @@ __device__ __forceinline__ Pair<P> load_pair(const ObsArgs<P>& a, int comp, long
 // precision (FP32 states: products of two stored floats) and accumulated per
 // thread (SumOf), then in FP64 per warp (shuffles), per block and over the
 // blocks, in a fixed order, so the result is deterministic for a given grid.
-// Plane-wave link factors c - i s come from a table: the cross term of a value
-// is c P + s Q with P = Re conj(G) (up - dn) and Q = Re -i conj(G) (up + dn) in
-// the state's precision.  kLink: LINK_TABLE is the quads' table of factors; any
+// Plane-wave link factors c - i s come from a table.  kLink: LINK_TABLE is the quads' table of factors; any
 // other vector potential (LINK_GENERAL) evaluates its phases in FP64.
 // Bound: loads (14 16-byte records per cell, about 5 from L2 or HBM).
 // us at 128^3 free / 4096^2 / 512^3 laser: with a block per 32 x 8 cells and z
@@ -212,7 +206,6 @@ __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
           zd = load_pair<P, kQuads>(a, 1, cell + (z == 0 ? nxy * Nz - nxy : -nxy));
         }
       }
-      R wP[2], wQ[2];
 #pragma unroll
       for (int l = 0; l < 2; ++l) {
         const int plane = 2 * c + l;
@@ -226,17 +219,21 @@ __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
           C up = ax == 0 ? (own_up ? q.v[l] : xp) : (ax == 1 ? (l == 0 ? q.v[1] : yp0) : zu.v[l]);
           C dn = ax == 0 ? (own_up ? xm : q.v[l]) : (ax == 1 ? (l == 0 ? ym1 : q.v[0]) : zd.v[l]);
           R re, im;
-          if (kLink == LINK_PLANE && ax == a.f.Apw_pol) {  // (the wave is across its own links: one factor for both)
-            const R dr = up.x - dn.x, di = up.y - dn.y, qr = up.x + dn.x, qi = up.y + dn.y;
-            // s_a with s_x = 1; s_y = -i (p=0) / +i (p=1); s_z = +1 (p=0) / -1 (p=1),
-            // applied to both parts: conj(G) s_a (D) and conj(G) s_a (-i Q)
-            const R sdr = ax == 1 ? (p ? -di : di) : (ax == 2 && p ? -dr : dr);
-            const R sdi = ax == 1 ? (p ? dr : -dr) : (ax == 2 && p ? -di : di);
-            const R sqr = ax == 1 ? (p ? qr : -qr) : (ax == 2 && p ? -qi : qi);
-            const R sqi = ax == 1 ? (p ? qi : -qi) : (ax == 2 && p ? qr : -qr);
-            wP[l] = G.x * sdr + G.y * sdi;
-            wQ[l] = G.x * sqr + G.y * sqi;
-            continue;
+          if (kLink == LINK_PLANE && ax == a.f.Apw_pol) {
+            // (the wave is across its own links: one factor c - i s for both, at
+            // the value's half-lattice coordinate along the wave vector)
+            const int h = a.wave_axis == 0 ? (int)H[0] : (a.wave_axis == 1 ? (int)H[1] : (int)H[2]);
+            if constexpr (sizeof(R) == 4) {
+              const float4 f = __ldg(&(static_cast<const PlaneLink32*>(a.wave) + h)->v);
+              const F32::Link L{make_float2(f.x, -f.z), make_float2(f.y, -f.w)};
+              const C w = rotated_diff(L, up, L, dn);
+              re = w.x;
+              im = w.y;
+            } else {
+              const double2 f = __ldg(static_cast<const double2*>(a.wave) + h);  // (cos phi, -sin phi)
+              re = f.x * (up.x - dn.x) - f.y * (up.y + dn.y);
+              im = f.x * (up.y - dn.y) + f.y * (up.x + dn.x);
+            }
           } else if (kLink == LINK_GENERAL) {
             const double2 u = mul_expm(widen(up), link_phase_site(a.f, DIMS, H, ax, +1, a.t_links, plane, cell));
             const double2 v = mul_expm(widen(dn), -link_phase_site(a.f, DIMS, H, ax, -1, a.t_links, plane, cell));
@@ -270,39 +267,10 @@ __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
           cb[ax] += G.x * sre + G.y * sim;  // Re(conj(G) s d)
         }
       }
-      if (kLink == LINK_PLANE) {
-        const int k = a.wave_axis;
-        const int o0 = plane_off<DIMS>(2 * c, 0), o1 = plane_off<DIMS>(2 * c, 1);
-        // half-lattice coordinate along the wave vector of each value (along z both are at the same level)
-        const int h0 = k == 0 ? 2 * x + o0 : (k == 1 ? 2 * yg + o1 : 2 * zg + plane_off<DIMS>(2 * c, 2));
-        const int h1 = k == 0 ? 2 * x + 1 - o0 : (k == 1 ? 2 * yg + 1 - o1 : h0);
-        // the wave's terms go to its polarisation axis
-        auto wave_term = [&](int h, R pt, R qt) {
-#pragma unroll
-          for (int ax = 0; ax < DIMS; ++ax) {  // (an index known at compile time)
-            if (ax != a.f.Apw_pol) continue;
-            if constexpr (sizeof(R) == 4) {
-              const float4 f = __ldg(&(static_cast<const PlaneLink32*>(a.wave) + h)->v);
-              sum[1 + ax].add_product(f.x, f.y, pt);
-              sum[1 + ax].add_product(f.z, f.w, qt);
-            } else {
-              const double2 f = __ldg(static_cast<const double2*>(a.wave) + h);  // (cos phi, -sin phi)
-              sum[1 + ax].add(f.x * pt - f.y * qt);
-            }
-          }
-        };
-        if (k == 2) {
-          wave_term(h0, wP[0] + wP[1], wQ[0] + wQ[1]);
-        } else {
-          wave_term(h0, wP[0], wQ[0]);
-          wave_term(h1, wP[1], wQ[1]);
-        }
-      }
     }
     sum[0].add(cn);
 #pragma unroll
-    for (int ax = 0; ax < DIMS; ++ax)
-      if (kLink != LINK_PLANE || ax != a.f.Apw_pol) sum[1 + ax].add(cb[ax]);
+    for (int ax = 0; ax < DIMS; ++ax) sum[1 + ax].add(cb[ax]);
     if (kDens) sum[4].add(cd);
     if (++pending == kFlush) {
       pending = 0;

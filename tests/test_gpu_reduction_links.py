@@ -53,3 +53,17 @@ def test_static_links(D, dims, N, precision, flags):
     prob = prob.with_fields(q=1.0, A_links=W.link_integrals(prob, lambda a, S, E: at(E) - at(S)))
     psi = np.stack([np.exp(1j * at(W.half_lattice_points(prob, p))) for p in range(prob.n_planes)])
     check(D, prob, psi, precision, flags)
+
+
+@pytest.mark.parametrize("precision,flags", [("fp64", 0), ("fp32", 0), ("fp32", 2)])
+@pytest.mark.parametrize("dims,N,along,pol", [(2, (31, 9, 1), 1, 0), (2, (65, 70, 1), 0, 1), (3, (33, 9, 7), 2, 0),
+                                              (3, (32, 12, 10), 0, 1), (3, (33, 9, 10), 1, 2)])
+def test_plane_wave(D, dims, N, along, pol, precision, flags):
+    """A wave so long that its phase is the same everywhere, 2 pi j over the period of the axis."""
+    prob = problem(dims, N)
+    phi = 2 * math.pi * max(1, N[pol] // 6) / (2 * N[pol])
+    k = [0.0, 0.0, 0.0]
+    k[along] = 1e-12
+    prob = prob.with_fields(q=1.0, Apw_amp=phi / (0.5 * prob.dx[pol]), Apw_k=tuple(k), Apw_pol=pol)
+    psi = np.stack([np.exp(1j * phi * W.half_lattice_points(prob, p)[pol]) for p in range(prob.n_planes)])
+    check(D, prob, psi, precision, flags)
