@@ -51,7 +51,10 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NS], double* out)
 // h goes to m, that of m to l (TwoSum, both exact), so only l rounds, by 2^-24 of
 // itself, at most 2^-64 of the largest partial sum over the kFlush cells after which
 // the three go to FP64.  FP64 additions one by one round by 2^-53 of the sum each.
+// Terms that kFlush of them could add up to beyond the floats' range, infinities
+// and NaN (which TwoSum would turn into NaN) go to FP64 by themselves.
 constexpr int kFlush = 16;
+constexpr float kSumMax = 0x1p120f;
 struct Sum32 {
   float h, m, l;
   // s becomes s + v, the result is what the rounding left out
@@ -268,10 +271,18 @@ __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
         }
       }
     }
-    sum[0].add(cn);
+    // (one test for all of a cell's terms; no density term exceeds cn)
+    if (sizeof(R) == 8 || fabs(cn) + (fabs(cb[0]) + fabs(cb[1]) + fabs(cb[2])) <= (R)kSumMax) {
+      sum[0].add(cn);
 #pragma unroll
-    for (int ax = 0; ax < DIMS; ++ax) sum[1 + ax].add(cb[ax]);
-    if (kDens) sum[4].add(cd);
+      for (int ax = 0; ax < DIMS; ++ax) sum[1 + ax].add(cb[ax]);
+      if (kDens) sum[4].add(cd);
+    } else {
+      acc[0] += cn;
+#pragma unroll
+      for (int ax = 0; ax < DIMS; ++ax) acc[1 + ax] += cb[ax];
+      if (kDens) acc[4] += cd;
+    }
     if (++pending == kFlush) {
       pending = 0;
 #pragma unroll

@@ -38,3 +38,25 @@ def test_terms_of_three_magnitudes(D, precision, flags):
         E, naive = s.norm()
         assert abs(naive - total) <= tol and abs(E - total) <= tol
         assert abs(s.partial_density(0, -1.0) - total) <= tol
+
+
+@pytest.mark.parametrize("flags", [0, 2])
+def test_sums_beyond_the_floats_range(D, flags):
+    """Squares that a float holds and their sums do not, and an infinite and a NaN value in one cell."""
+    prob = W.Problem(2, (32, 80000, 1), (1.0, 1.0, 1.0), 0.6, 0.4)
+    psi = np.zeros(prob.shape, dtype=np.complex128)
+    v = float(np.float32(1.5e19))
+    psi[0] = v
+    n = psi[0].size
+    with D.Sim(prob, D.FP32, flags=flags) as s:
+        s.set_spinor(psi)
+        _, naive = s.norm()
+        # every square is rounded once, to 2^-24 of itself
+        assert abs(naive - n * v * v) <= 2.0 ** -24 * n * v * v
+        for bad in (np.inf, np.nan):
+            psi[0, 0, 41234, 7] = bad
+            s.set_spinor(psi)
+            n = s.partial_density(0, -1.0)
+            assert np.isinf(n) and n > 0 if np.isinf(bad) else np.isnan(n)
+            with pytest.raises(D.DiracError):  # a functional that is not finite is reported
+                s.norm()
