@@ -73,6 +73,7 @@ struct dirac_sim {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   void* graph_state[2] = {nullptr, nullptr};
   long long graph_launches[2] = {0, 0};  // kernels in each
+  int graph_swaps[2] = {0, 0};           // its passes leave the state in the other buffer
   int graph_disabled = 0;
   int stepped = 0;            // a plain step has run (kernel one-time set-up done)
   // conserved functional accumulated by the last fused launch of a dirac_step
@@ -1162,6 +1163,7 @@ static dirac_status build_graph(dirac_sim* s, int slot) {
   }
   // capturing did not run anything: restore the bookkeeping
   s->graph_launches[slot] = s->launches - l0;
+  s->graph_swaps[slot] = s->state != state0;
   s->k = k0;
   s->launches = l0;
   if (s->state != state0) std::swap(s->state, s->state_alt);
@@ -1207,7 +1209,7 @@ extern "C" dirac_status dirac_step(dirac_sim* s, long nsteps) {
     CK(s, cudaGraphLaunch(s->graph[slot], s->stream));
     s->launches += s->graph_launches[slot];
     s->k += kGraphSteps;
-    if (s->fused && (s->graph_launches[slot] & 1)) std::swap(s->state, s->state_alt);
+    if (s->graph_swaps[slot]) std::swap(s->state, s->state_alt);
     nsteps -= kGraphSteps;
   }
   return steps_plain(s, nsteps, s->stream, true);

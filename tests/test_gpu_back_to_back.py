@@ -59,3 +59,14 @@ def test_hundreds_of_launches_over_a_state_in_cache(D, monkeypatch, graphs, dims
     prob = W.Problem(dims, N, (1.0, 1.0, 1.0), 0.9 * W.stability_limit(dims), 0.4, W.Fields(**f))
     psi = W.random_state(prob, 23)
     assert np.array_equal(run(D, prob, psi, 401), run(D, prob, psi, 401, flags=D.FLAG_REFERENCE_KERNELS))
+
+
+@pytest.mark.parametrize("n", [129, 194, 260])
+@pytest.mark.parametrize("N", [(40, 200), (24, 2800)])
+def test_graph_replays_with_link_tables(D, N, n):
+    """A plane wave that does not move: its link tables are formed inside the graphs of 64 steps,
+    and whatever their number the passes alone decide where the state ends up."""
+    f = W.Fields(q=1.0, Apw_amp=0.5, Apw_k=(0.0, 2 * math.pi / N[1], 0.0), Apw_pol=0)
+    prob = W.Problem(2, (N[0], N[1], 1), (1.0, 1.0, 1.0), 0.6, 0.4, f)
+    psi = W.random_state(prob, 29)
+    assert np.array_equal(run(D, prob, psi, n), run(D, prob, psi, n, flags=D.FLAG_REFERENCE_KERNELS))
