@@ -328,11 +328,13 @@ struct LinkTimes {
 template <class P>
 __global__ void link_table_kernel(typename PlaneLinkOf<P>::type* tab, int n, const FieldDesc f, int dims,
                                   int axis, int pol, const LinkTimes t, int steps) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 2 * n * steps) return;
-  const int step = i / (2 * n), j = i - step * 2 * n, half = j / n;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x, per_step = 2LL * n;
+  if (i >= per_step * steps) return;
+  const int step = (int)(i / per_step);
+  const long long j = i - step * per_step;
+  const int half = j >= n;
   long long HH[3] = {0, 0, 0};
-  HH[axis] = j - half * n;
+  HH[axis] = half ? j - n : j;
   // the same phase function as the per-link FP64 path
   plane_link_from(link_phase(f, dims, HH, pol, +1, half ? t.lo[step] : t.up[step]), tab + i);
 }
@@ -653,7 +655,7 @@ void launch_link_table(void* tab, int n, const FieldDesc& f, int dims, int axis,
     t.up[j] = t_up[j];
     t.lo[j] = t_lo[j];
   }
-  link_table_kernel<P><<<(2 * n * steps + 127) / 128, 128, 0, s>>>(
+  link_table_kernel<P><<<(unsigned)((2LL * n * steps + 127) / 128), 128, 0, s>>>(
       static_cast<typename PlaneLinkOf<P>::type*>(tab), n, f, dims, axis, pol, t, steps);
 }
 template void launch_link_table<F64>(void*, int, const FieldDesc&, int, int, int, const double*, const double*, int,
