@@ -364,7 +364,10 @@ double dirac_algorithmic_bytes(const dirac_sim* sim);
    (DIRAC_FP32, time-independent) or 32 (DIRAC_FP64, time-independent, where
    that leaves at least as much device memory free), A_links 16 bytes per axis and value, a
    tabulated static vector potential (DIRAC_FP32) 32 bytes per axis and
-   value, and every simulation a few KiB of reduction scratch. */
+   value, a plane wave whose wave vector lies along one axis other than its
+   polarisation the link factors of 32 steps, 256 bytes (DIRAC_FP64: 64) per
+   step and cell along the wave (of fewer steps where they would exceed both
+   16 MiB and a quarter of the state's buffers; one at least), and every simulation a few KiB of reduction scratch. */
 size_t dirac_state_bytes(int dims, const int N[3], dirac_precision precision);
 
 /* human-readable description of the last failure on sim (or, when sim is

@@ -63,9 +63,9 @@ struct dirac_sim {
   int iso = 1;
   int coef_mode = COEF_UNIFORM, link_mode = LINK_NONE;
   int step_X = 0;
-  void* ltab = nullptr;       // LINK_PLANE: link-factor tables of kTableSteps steps
+  void* ltab = nullptr;       // LINK_PLANE: link-factor tables of ltab_steps steps, or of a reduction's time
   int ltab_step = 0;          // the current step's among them
-  void* wave = nullptr;       // LINK_PLANE: link-factor table of the reductions
+  int ltab_steps = 0;
   int ltab_axis = 0, ltab_n = 0;
   long long launches = 0;     // kernels launched so far
   // CUDA graphs of kGraphSteps time steps, one per current-buffer parity
@@ -794,10 +794,14 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
     s->launches += 1;
   }
   if (s->link_mode == LINK_PLANE) {
-    const size_t tb = (size_t)2 * kTableSteps * s->ltab_n *
-                      (precision == DIRAC_FP32 ? sizeof(PlaneLinkOf<F32>::type) : sizeof(PlaneLinkOf<F64>::type));
-    if ((e = cudaMalloc(&s->ltab, tb)) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link table)"));
-    if ((e = cudaMalloc(&s->wave, tb / kTableSteps)) != cudaSuccess)
+    // as many steps per table launch as a quarter of the state holds, or 16 MiB (32
+    // steps up to 2048 cells along the wave), and at least one: a grid long
+    // along the wave and narrow across it would have more table than state
+    const size_t step = (size_t)2 * s->ltab_n *
+                        (precision == DIRAC_FP32 ? sizeof(PlaneLinkOf<F32>::type) : sizeof(PlaneLinkOf<F64>::type));
+    const size_t most = std::max(sbytes / 4 * (s->fused ? 2 : 1), (size_t)16 << 20) / step;
+    s->ltab_steps = most >= (size_t)kTableSteps ? kTableSteps : (most < 2 ? 1 : (int)most & ~1);  // (whole passes)
+    if ((e = cudaMalloc(&s->ltab, s->ltab_steps * step)) != cudaSuccess)
       return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link table)"));
   }
   if (s->fused) {
@@ -848,7 +852,6 @@ extern "C" void dirac_destroy(dirac_sim* s) {
   cudaFree(s->Alink);
   cudaFree(s->larr);
   cudaFree(s->ltab);
-  cudaFree(s->wave);
   cudaFree(s->e_partials);
   cudaFree(s->e_sums);
   cudaFree(s->partials);
@@ -1037,7 +1040,7 @@ static bool time_dependent_fields(const dirac_sim* s) {
 static double time_after(const dirac_sim* s, long long steps) { return s->t0 + (double)(s->k + steps) * s->dt; }
 
 // LINK_PLANE: the link-factor tables (both half-steps) of a run of n time steps,
-// kTableSteps of them per launch: begin() before each pass of `steps` steps
+// ltab_steps of them per launch: begin() before each pass of `steps` steps
 // with n steps left to go (itself included).  A launch per step cost a (2+1)D pass
 // 9 % of its time (1000^2: 16.6 us per step, now 13.5).
 template <class P>
@@ -1046,7 +1049,7 @@ struct LinkTables {
   void begin(dirac_sim* s, int steps, long n, cudaStream_t st) {
     if (s->link_mode != LINK_PLANE) return;
     if (have < steps) {
-      have = n < kTableSteps ? n : kTableSteps;
+      have = n < s->ltab_steps ? n : s->ltab_steps;
       double up[kTableSteps], lo[kTableSteps];
       for (int j = 0; j < (int)have; ++j) {
         up[j] = time_after(s, j);
@@ -1100,7 +1103,7 @@ static bool per_site_path(const dirac_sim* s) {
 // table per step); the grid needs four rows.
 static int steps_per_pass(const dirac_sim* s, long n) {
   const bool whole = s->zlo == 0 && s->zorg == 0 && s->nzu == s->Nzg;
-  if (s->dims != 2 || !s->tblock || !whole || per_site_path(s) ||
+  if (s->dims != 2 || !s->tblock || !whole || per_site_path(s) || (s->link_mode == LINK_PLANE && s->ltab_steps < 2) ||
       std::getenv("DIRAC_NO_TEMPORAL_BLOCKING") != nullptr)
     return 1;
   return n >= 2 && s->N[1] >= 4 ? 2 : 1;
@@ -1507,11 +1510,11 @@ static dirac_status observe_launch(dirac_sim* s, int dens_axis, int dens_X, doub
   a.f = field_desc(s);
   a.t_links = sim_time(s) - s->dt / 2.0;
   if (s->link_mode == LINK_PLANE) {
-    launch_link_table<P>(s->wave, s->ltab_n, a.f, s->dims, s->ltab_axis, s->f.Apw_pol, &a.t_links, &a.t_links, 1,
+    launch_link_table<P>(s->ltab, s->ltab_n, a.f, s->dims, s->ltab_axis, s->f.Apw_pol, &a.t_links, &a.t_links, 1,
                          s->stream);
     s->launches += 1;
     CK(s, cudaGetLastError());
-    a.wave = s->wave;
+    a.wave = s->ltab;  // (every call that steps forms its tables anew)
     a.wave_axis = s->ltab_axis;
   }
   if (s->link_mode == LINK_TABLE && s->fused) a.lq = static_cast<const float4*>(s->larr);

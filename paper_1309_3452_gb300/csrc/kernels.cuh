@@ -82,7 +82,7 @@ constexpr int kFusedEMaxBlocks = 4096;  // capacity of the per-block E partials
 // (2+1)D fused kernel geometry
 constexpr int kFused2dWarps = 4;   // independent x strips per block (few, so that small grids spread over the SMs)
 constexpr int kMaxSteps2d = 2;     // most time steps per pass
-constexpr int kTableSteps = 32;    // time steps whose plane-wave link tables one launch forms
+constexpr int kTableSteps = 32;    // most time steps whose plane-wave link tables one launch forms
 
 // returns the number of blocks launched
 template <class P, int DIMS>

@@ -1,6 +1,7 @@
 """The plane waves' link tables on grids long along the wave."""
 import math
 
+import numpy as np
 import pytest
 
 from paper_1309_3452_gb300 import workloads as W
@@ -38,3 +39,31 @@ def test_2_to_the_31_table_entries(D):
             s.get_spinor_device(out[-1].data_ptr())
             torch.cuda.synchronize()
     assert torch.equal(out[0], out[1])
+
+
+def test_memory_of_a_grid_long_along_the_wave(D):
+    """One step's factors (256 bytes per cell along the wave) where a quarter of the state holds no more."""
+    import torch
+    prob = problem((1 << 20, 8, 1))
+    with D.Sim(prob, D.FP32) as s:  # (whatever the library allocates once)
+        pass
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    with D.Sim(prob, D.FP32) as s:
+        used = free0 - torch.cuda.mem_get_info()[0]
+    assert used <= D.state_bytes(2, prob.N, D.FP32) + (256 << 20) + (64 << 20)  # (allocations come in 2 MiB pages)
+
+
+@pytest.mark.parametrize("N", [(40000, 8), (20000, 5), (70000, 4), (2500, 9)])
+def test_tables_of_fewer_steps(D, N):
+    """1, 2 and 26 steps per table; 67 steps, so that tables, passes and calls end at different steps."""
+    prob = problem((N[0], N[1], 1))
+    psi = W.random_state(prob, 37)
+    out = []
+    for flags in (0, D.FLAG_REFERENCE_KERNELS):
+        with D.Sim(prob, D.FP32, flags=flags) as s:
+            s.set_spinor(psi)
+            s.step(40)
+            s.step(27)
+            out.append(s.get_spinor())
+    assert np.array_equal(out[0], out[1])
