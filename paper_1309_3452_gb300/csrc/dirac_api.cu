@@ -51,6 +51,7 @@ struct dirac_sim {
   F64::Coef* c_tab = nullptr; // COEF_TABLE, FP64: alpha and gamma per site (plane-major, pstride)
   unsigned* sc_corr = nullptr; // COEF_SOFTCORR: one 32-bit correction word per value
   double* Alink = nullptr;    // link integrals x q: 2 dims slots (up, down link per axis) of np * pstride
+                              // (LINK_UP: up links alone, and only until the factors are formed)
   void* larr = nullptr;       // LINK_TABLE, LINK_UP: link factors (F32::Link, FP64: F64::Link)
   double* partials = nullptr;
   double* sums_dev = nullptr;
@@ -281,7 +282,7 @@ static FieldDesc field_desc(const dirac_sim* s) {
   d.abs_axes = s->f.abs_axes;
   for (int a = 0; a < 3; ++a) d.L[a] = s->Nf[a] * s->dx[a];
   d.Alink = s->Alink;
-  d.Alink_n = (long long)s->np * s->pstride;
+  d.Alink_n = (long long)s->np * s->pstride / (s->link_mode == LINK_UP ? 2 : 1);  // (slot 2a is the a-th array there)
   d.Alink_ps = s->pstride;
   d.Alink_amp = s->f.Alink_amp;
   d.Alink_omega = s->f.Alink_omega;
@@ -623,7 +624,8 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
   // tabulated once for the FP32 kernels instead of a sincos per link and step
   const bool moving = (f.Apw_amp != 0.0 && f.Apw_omega != 0.0) ||
                       (alinks && f.Alink_amp != 0.0 && f.Alink_omega != 0.0);
-  // (FP64: where it is given by its link integrals alone and the memory allows it)
+  // (FP64: where it is given by its link integrals alone: the up links' factors
+  // take the room that both links' integrals would)
   if (s->link_mode == LINK_GENERAL && !moving) {
     if (precision == DIRAC_FP32) s->link_mode = LINK_TABLE;
     else if (alinks && f.Apw_amp == 0.0) s->link_mode = LINK_UP;
@@ -662,7 +664,8 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
   }
   if (alinks) {
     const size_t per_axis = (size_t)s->np * s->ncell;
-    const size_t tb = (size_t)2 * dims * s->np * s->pstride * sizeof(double);
+    const int dirs = s->link_mode == LINK_UP ? 1 : 2;
+    const size_t tb = (size_t)dirs * dims * s->np * s->pstride * sizeof(double);
     if ((e = cudaMalloc(&s->Alink, tb)) != cudaSuccess)
       return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link integrals)"));
     if ((e = cudaMemsetAsync(s->Alink, 0, tb, s->stream)) != cudaSuccess)
@@ -672,7 +675,7 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
       return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link integrals, upload)"));
     e = cudaMemcpyAsync(raw, f.A_links, dims * per_axis * sizeof(double), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess) {
-      launch_link_integral_table(s->Alink, raw, dims, s->N, s->pstride, f.q, s->stream);
+      launch_link_integral_table(s->Alink, raw, dims, s->N, s->pstride, f.q, dirs, s->stream);
       e = cudaGetLastError();
       s->launches += 1;
     }
@@ -684,32 +687,23 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
     const int dirs = s->link_mode == LINK_UP ? 1 : 2;
     const size_t tb = (size_t)dirs * dims * s->np * s->pstride * sizeof(F32::Link);
     static_assert(sizeof(F32::Link) == sizeof(F64::Link), "one size for both precisions");
-    if (precision == DIRAC_FP64) {  // where the table leaves as much device memory as it takes, else per site
-      size_t mem_free = 0, mem_total = 0;
-      if ((e = cudaMemGetInfo(&mem_free, &mem_total)) != cudaSuccess)
-        return cleanup_fail(cuda_fail(s, e, "cudaMemGetInfo"));
-      e = tb <= mem_free / 2 ? cudaMalloc(&s->larr, tb) : cudaErrorMemoryAllocation;
-      if (e == cudaErrorMemoryAllocation) {
-        s->larr = nullptr;
-        cudaGetLastError();  // not an error of this simulation
-        s->link_mode = LINK_GENERAL;
-        e = cudaSuccess;
-      }
-    } else {
-      e = cudaMalloc(&s->larr, tb);
-    }
-    if (e != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link factor table)"));
-    if (s->larr) {
-      if ((e = cudaMemsetAsync(s->larr, 0, tb, s->stream)) != cudaSuccess)
-        return cleanup_fail(cuda_fail(s, e, "cudaMemsetAsync(link factor table)"));
-      if (precision == DIRAC_FP64)
-        launch_link_factor_table<F64>(static_cast<F64::Link*>(s->larr), field_desc(s), dims, s->N, s->pstride, 0, dirs,
-                                      s->stream);
-      else
-        launch_link_factor_table<F32>(static_cast<F32::Link*>(s->larr), field_desc(s), dims, s->N, s->pstride,
-                                      s->fused, dirs, s->stream);
-      if ((e = cudaGetLastError()) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "link factor table"));
-      s->launches += 1;
+    if ((e = cudaMalloc(&s->larr, tb)) != cudaSuccess)
+      return cleanup_fail(cuda_fail(s, e, "cudaMalloc(link factor table)"));
+    if ((e = cudaMemsetAsync(s->larr, 0, tb, s->stream)) != cudaSuccess)
+      return cleanup_fail(cuda_fail(s, e, "cudaMemsetAsync(link factor table)"));
+    if (precision == DIRAC_FP64)
+      launch_link_factor_table<F64>(static_cast<F64::Link*>(s->larr), field_desc(s), dims, s->N, s->pstride, 0, dirs,
+                                    s->stream);
+    else
+      launch_link_factor_table<F32>(static_cast<F32::Link*>(s->larr), field_desc(s), dims, s->N, s->pstride,
+                                    s->fused, dirs, s->stream);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "link factor table"));
+    s->launches += 1;
+    if (s->link_mode == LINK_UP) {
+      if ((e = cudaStreamSynchronize(s->stream)) != cudaSuccess)
+        return cleanup_fail(cuda_fail(s, e, "link factor table"));
+      cudaFree(s->Alink);
+      s->Alink = nullptr;
     }
   }
   if (s->coef_mode == COEF_SOFTCORE || s->coef_mode == COEF_SOFTCORR) {
@@ -1795,7 +1789,8 @@ extern "C" double dirac_algorithmic_bytes(const dirac_sim* s) {
   if (s->coef_mode == COEF_SOFTCORR) b += 4.0 * s->np;         // one correction word per value read
   if ((s->coef_mode == COEF_GENERAL && s->Vstatic) || (s->c_tab && s->vstatic)) b += 8.0 * s->np;  // one real per value
   if (s->link_mode == LINK_TABLE) b += 32.0 * s->dims * s->np;  // up and down link factor (hi + lo) per axis
-  else if (s->Alink) b += 16.0 * s->dims * s->np;              // up and down link integral per axis
+  else if (s->Alink || s->link_mode == LINK_UP)
+    b += 16.0 * s->dims * s->np;                               // up and down link integral (or an up factor) per axis
   return b;
 }
 

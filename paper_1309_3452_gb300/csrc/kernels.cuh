@@ -182,9 +182,10 @@ void launch_softcore_corr(unsigned* out, const HalfFields<F32>& hu, const HalfFi
 // link integrals of an arbitrary vector potential (Sect. 4): raw = the
 // caller's integrals [axis][plane][cell] (canonical layout, cells dense), out
 // = q times them per value in the state layout, slot 2a = the value's up link
-// and 2a+1 = its down link: out[slot * P * pstride + plane * pstride + cell]
+// and 2a+1 = its down link (dirs = 1: slot a, the up link alone):
+// out[slot * P * pstride + plane * pstride + cell]
 void launch_link_integral_table(double* out, const double* raw, int dims, const int N[3], long long pstride,
-                                double q, cudaStream_t s);
+                                double q, int dirs, cudaStream_t s);
 
 // exp(-i phi) of every value's links of a time-independent vector potential:
 // out[slot * P * pstride + plane * pstride + cell], or (quads, F32) the quad

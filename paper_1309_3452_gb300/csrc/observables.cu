@@ -435,12 +435,12 @@ __global__ void softcore_corr_kernel(unsigned* __restrict__ out, const HalfField
 }
 
 // q times the link integrals of every value in the state layout: the value's
-// own link towards +dx_a/2 (slot 2a) and the link from its neighbour at
+// own link towards +dx_a/2 (slot 2a; alone, dirs = 1: slot a) and the link from its neighbour at
 // -dx_a/2 to it (slot 2a+1), which that neighbour (partner plane, cell shifted
 // with the periodic wrap) carries as its own up link
 template <int DIMS>
 __global__ void link_integral_table_kernel(double* __restrict__ out, const double* __restrict__ raw, int N0,
-                                           int N1, int N2, long long pstride, double q) {
+                                           int N1, int N2, long long pstride, double q, int dirs) {
   const int plane = blockIdx.y, axis = blockIdx.z;
   const long long ncell = (long long)N0 * N1 * N2;
   const long long n = (long long)nplanes<DIMS>() * pstride;
@@ -455,8 +455,8 @@ __global__ void link_integral_table_kernel(double* __restrict__ out, const doubl
     long long jm = j[axis] + shift;
     if (jm < 0) jm += Nn[axis];
     const long long cm = c + (jm - j[axis]) * stride[axis];
-    out[(2LL * axis) * n + plane * pstride + c] = q * raw_a[(long long)plane * ncell + c];
-    out[(2LL * axis + 1) * n + plane * pstride + c] = q * raw_a[(long long)pp * ncell + cm];
+    out[(long long)(dirs * axis) * n + plane * pstride + c] = q * raw_a[(long long)plane * ncell + c];
+    if (dirs == 2) out[(2LL * axis + 1) * n + plane * pstride + c] = q * raw_a[(long long)pp * ncell + cm];
   }
 }
 
@@ -699,15 +699,15 @@ void launch_softcore_corr(unsigned* out, const HalfFields<F32>& hu, const HalfFi
 }
 
 void launch_link_integral_table(double* out, const double* raw, int dims, const int N[3], long long pstride,
-                                double q, cudaStream_t s) {
+                                double q, int dirs, cudaStream_t s) {
   const long long ncell = (long long)N[0] * N[1] * (dims == 3 ? N[2] : 1);
   long long bx = (ncell + 255) / 256;
   if (bx > 152 * 16) bx = 152 * 16;
   const dim3 grid((unsigned)bx, dims == 3 ? 8 : 4, dims);
   if (dims == 3)
-    link_integral_table_kernel<3><<<grid, 256, 0, s>>>(out, raw, N[0], N[1], N[2], pstride, q);
+    link_integral_table_kernel<3><<<grid, 256, 0, s>>>(out, raw, N[0], N[1], N[2], pstride, q, dirs);
   else
-    link_integral_table_kernel<2><<<grid, 256, 0, s>>>(out, raw, N[0], N[1], 1, pstride, q);
+    link_integral_table_kernel<2><<<grid, 256, 0, s>>>(out, raw, N[0], N[1], 1, pstride, q, dirs);
 }
 
 template <class P>
