@@ -362,7 +362,9 @@ double dirac_algorithmic_bytes(const dirac_sim* sim);
    Other potentials add one double per value (a static array that DIRAC_FP64
    or a time dependence keeps) and the coefficient table, 16 bytes per value
    (DIRAC_FP32, time-independent) or 32 (DIRAC_FP64, time-independent, where
-   that leaves at least as much device memory free), A_links 16 bytes per axis and value, a
+   that leaves at least as much device memory free and all such tables take
+   at most an eighth of it; a simulation that does not fit otherwise is given
+   those of others, whose values stay the same), A_links 16 bytes per axis and value, a
    tabulated static vector potential (DIRAC_FP32) 32 bytes per axis and
    value, a plane wave whose wave vector lies along one axis other than its
    polarisation the link factors of 32 steps, 256 bytes (DIRAC_FP64: 64) per

@@ -43,12 +43,17 @@ struct dirac_sim {
   double plan_us = 0;         // time per step the autotuner measured for the plan
   double2* staging = nullptr; // one canonical plane (FP32 conversions)
   double* Vstatic = nullptr;  // one real per site (plane-major, pstride)
-  int vstatic = 0;            // the caller gave a static array (which a table may have replaced)
   float4* b_tab = nullptr;    // COEF_TABLE: b = 1/(1 + i theta) per site as hi + lo (plane-major, pstride)
   unsigned* b_map = nullptr;  // fused kernels: the cells' classes in b_tab, and a cell of each (HalfFields::b_map)
   long long b_ps = 0;         // classes (b_tab's records per component)
   float2* sc_sq = nullptr;    // COEF_SOFTCORE/CORR: (X dx_a/2 - c_a)^2 per axis and half-lattice index, hi + lo
-  F64::Coef* c_tab = nullptr; // COEF_TABLE, FP64: alpha and gamma per site (plane-major, pstride)
+  // COEF_TABLE, FP64: alpha and gamma per site (plane-major, pstride).  Another
+  // simulation's creation may take it back (release_coef_tables): c_mu is held where
+  // launches that read it are made
+  F64::Coef* c_tab = nullptr;
+  mutable std::mutex c_mu;
+  int c_kept = 0;             // a caller's capture has recorded it: never taken back
+  int dev = 0;                // the device it was created on
   unsigned* sc_corr = nullptr; // COEF_SOFTCORR: one 32-bit correction word per value
   double* Alink = nullptr;    // link integrals x q: 2 dims slots (up, down link per axis) of np * pstride
                               // (LINK_UP: up links alone, and only until the factors are formed)
@@ -464,6 +469,58 @@ static void drop_graphs(dirac_sim* s) {
   }
 }
 
+// The FP64 coefficient tables (32 bytes per value beside a state of 16): none that
+// a program could miss is kept.  All together they take at most an eighth of the
+// device, so that other allocations of the process find most of it, and where
+// a simulation's own allocations do not fit, the tables of the others go first:
+// their potential is evaluated per site from then on (the same values).
+struct CoefTables {
+  std::mutex mu;                  // guards what follows; taken before a simulation's c_mu
+  std::vector<dirac_sim*> sims;   // the simulations that have one
+};
+static CoefTables g_coef;
+
+static size_t coef_table_bytes(const dirac_sim* s) { return (size_t)s->np * s->pstride * sizeof(F64::Coef); }
+
+// room for this simulation's table; *e: a failed query
+static bool coef_table_fits(const dirac_sim* s, cudaError_t* e) {
+  size_t mem_free = 0, mem_total = 0;
+  if ((*e = cudaMemGetInfo(&mem_free, &mem_total)) != cudaSuccess) return false;
+  const size_t need = coef_table_bytes(s);
+  size_t held = need;
+  std::lock_guard<std::mutex> lock(g_coef.mu);
+  for (const dirac_sim* o : g_coef.sims)
+    if (o->dev == s->dev) held += coef_table_bytes(o);
+  return need <= mem_free / 2 && held <= mem_total / 8;
+}
+
+// Take back the current device's tables; true if one went.
+static bool release_coef_tables() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> lock(g_coef.mu);
+  bool any = false;
+  auto keeps = [&](dirac_sim* s) {
+    std::lock_guard<std::mutex> hold(s->c_mu);  // (a call that steps it ends first)
+    if (s->c_kept || s->dev != dev) return true;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
+        cudaStreamSynchronize(s->stream) != cudaSuccess) {
+      cudaGetLastError();  // that simulation's own calls report it
+      return true;
+    }
+    drop_graphs(s);
+    cudaFree(s->c_tab);
+    s->c_tab = nullptr;
+    s->coef_mode = COEF_GENERAL;
+    any = true;
+    return false;
+  };
+  g_coef.sims.erase(std::remove_if(g_coef.sims.begin(), g_coef.sims.end(), [&](dirac_sim* s) { return !keeps(s); }),
+                    g_coef.sims.end());
+  return any;
+}
+
 static dirac_plan plan_of(const dirac_sim* s) {
   dirac_plan p;
   std::memset(&p, 0, sizeof(p));
@@ -504,6 +561,9 @@ struct SlabSpec {
 static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const double dx[3], double dt,
                                double m, const dirac_fields* fields, dirac_precision precision, unsigned flags,
                                void* stream, const SlabSpec& slab);
+static dirac_status create_once(dirac_sim** out, int dims, const int N[3], const double dx[3], double dt,
+                                double m, const dirac_fields* fields, dirac_precision precision, unsigned flags,
+                                void* stream, const SlabSpec& slab);
 
 extern "C" dirac_status dirac_create(dirac_sim** out, int dims, const int N[3], const double dx[3],
                                      double dt, double m, const dirac_fields* fields,
@@ -514,6 +574,14 @@ extern "C" dirac_status dirac_create(dirac_sim** out, int dims, const int N[3], 
 static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const double dx[3], double dt,
                                double m, const dirac_fields* fields, dirac_precision precision, unsigned flags,
                                void* stream, const SlabSpec& slab) {
+  const dirac_status st = create_once(out, dims, N, dx, dt, m, fields, precision, flags, stream, slab);
+  if (st != DIRAC_ERR_OOM || !release_coef_tables()) return st;
+  return create_once(out, dims, N, dx, dt, m, fields, precision, flags, stream, slab);
+}
+
+static dirac_status create_once(dirac_sim** out, int dims, const int N[3], const double dx[3], double dt,
+                                double m, const dirac_fields* fields, dirac_precision precision, unsigned flags,
+                                void* stream, const SlabSpec& slab) {
   if (!out) return fail(nullptr, DIRAC_ERR_INVALID, "out is NULL");
   *out = nullptr;
   if (dims != 2 && dims != 3) return fail(nullptr, DIRAC_ERR_INVALID, "dims must be 2 or 3");
@@ -563,6 +631,7 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
   s->f.V_static = nullptr;
   s->f.A_links = nullptr;
   s->stream = static_cast<cudaStream_t>(stream);
+  cudaGetDevice(&s->dev);
   for (int a = 0; a < 3; ++a) s->Nf[a] = s->N[a];
   const int march = dims == 3 ? 2 : 1;  // the fused kernels' marching axis
   if (slab.on) {  // N is the whole grid: store the slab's levels and two halo levels
@@ -585,7 +654,6 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
   // a time-independent potential beyond V0 and the step: tabulated for the FP32
   // kernels, evaluated per site in FP64 otherwise
   const bool vstatic = fields && fields->V_static;
-  s->vstatic = vstatic;
   const bool layers = f.abs_W != 0.0;
   // a real soft core (with V0 and a Klein step, nothing else): analytic per
   // value in the FP32 kernels, no per-site data
@@ -743,13 +811,11 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
   }
   if (s->coef_mode == COEF_GENERAL && !(s->Vstatic && f.Vmod_amp != 0.0)) {
     // FP64, a potential that does not change in time: tabulated where the table
-    // leaves the caller as much free device memory as it takes, else evaluated
-    // per site (same values)
-    const size_t tb = (size_t)s->np * s->pstride * sizeof(F64::Coef);
-    size_t mem_free = 0, mem_total = 0;
-    if ((e = cudaMemGetInfo(&mem_free, &mem_total)) != cudaSuccess)
-      return cleanup_fail(cuda_fail(s, e, "cudaMemGetInfo"));
-    e = tb <= mem_free / 2 ? cudaMalloc(&s->c_tab, tb) : cudaErrorMemoryAllocation;
+    // fits, else evaluated per site (same values)
+    e = cudaSuccess;
+    const bool fits = coef_table_fits(s, &e);
+    if (e != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "cudaMemGetInfo"));
+    e = fits ? cudaMalloc(&s->c_tab, coef_table_bytes(s)) : cudaErrorMemoryAllocation;
     if (e == cudaSuccess) {
       launch_coef64_table(s->c_tab, field_desc(s), dims, s->N, s->pstride, s->stream);
       if ((e = cudaGetLastError()) != cudaSuccess) return cleanup_fail(cuda_fail(s, e, "coefficient table"));
@@ -813,7 +879,7 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
     return cleanup_fail(cuda_fail(s, e, "cudaMallocHost(sums)"));
   if ((e = cudaStreamSynchronize(s->stream)) != cudaSuccess)
     return cleanup_fail(cuda_fail(s, e, "cudaStreamSynchronize"));
-  if (s->coef_mode == COEF_TABLE && s->Vstatic) {  // folded into the table
+  if (s->coef_mode == COEF_TABLE && s->Vstatic && !s->c_tab) {  // folded into the table for good
     cudaFree(s->Vstatic);
     s->Vstatic = nullptr;
   }
@@ -821,6 +887,10 @@ static dirac_status create_sim(dirac_sim** out, int dims, const int N[3], const 
     std::lock_guard<std::mutex> lock(g_plan_mu);
     auto it = g_plans.find(plan_key(s));
     if (it != g_plans.end()) apply_plan(s, it->second);
+  }
+  if (s->c_tab) {
+    std::lock_guard<std::mutex> lock(g_coef.mu);
+    g_coef.sims.push_back(s);
   }
   *out = s;
   return DIRAC_OK;
@@ -830,6 +900,10 @@ static void drop_batch_graphs(const dirac_sim* s);
 
 extern "C" void dirac_destroy(dirac_sim* s) {
   if (!s) return;
+  {
+    std::lock_guard<std::mutex> lock(g_coef.mu);
+    g_coef.sims.erase(std::remove(g_coef.sims.begin(), g_coef.sims.end(), s), g_coef.sims.end());
+  }
   cudaStreamSynchronize(s->stream);
   drop_batch_graphs(s);
   for (int k = 0; k < 2; ++k)
@@ -1187,6 +1261,13 @@ static dirac_status build_graph(dirac_sim* s, int slot) {
 extern "C" dirac_status dirac_step(dirac_sim* s, long nsteps) {
   if (!s) return fail(s, DIRAC_ERR_INVALID, "NULL sim");
   if (nsteps < 0) return fail(s, DIRAC_ERR_INVALID, "nsteps < 0");
+  std::unique_lock<std::mutex> hold(s->c_mu, std::defer_lock);
+  if (s->prec == DIRAC_FP64) {
+    hold.lock();
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (s->c_tab && cudaStreamIsCapturing(s->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive)
+      s->c_kept = 1;
+  }
   const bool graphs = !s->graph_disabled && !time_dependent_fields(s) &&
                       std::getenv("DIRAC_NO_GRAPHS") == nullptr;
   if (graphs && !s->stepped && nsteps > kGraphSteps) {
@@ -1782,12 +1863,13 @@ extern "C" dirac_status dirac_check(dirac_sim* s, double tol, dirac_check_report
 
 extern "C" double dirac_algorithmic_bytes(const dirac_sim* s) {
   if (!s) return 0.0;
+  std::lock_guard<std::mutex> hold(s->c_mu);
   double b = 2.0 * s->np * (double)s->elem;                    // every value read and written once
   // one coefficient per value read (FP64's table of alpha and gamma is the
   // library's choice: there the data given per site counts, below)
   if (s->coef_mode == COEF_TABLE && !s->c_tab) b += 16.0 * s->np;
   if (s->coef_mode == COEF_SOFTCORR) b += 4.0 * s->np;         // one correction word per value read
-  if ((s->coef_mode == COEF_GENERAL && s->Vstatic) || (s->c_tab && s->vstatic)) b += 8.0 * s->np;  // one real per value
+  if ((s->coef_mode == COEF_GENERAL || s->c_tab) && s->Vstatic) b += 8.0 * s->np;  // one real per value
   if (s->link_mode == LINK_TABLE) b += 32.0 * s->dims * s->np;  // up and down link factor (hi + lo) per axis
   else if (s->Alink || s->link_mode == LINK_UP)
     b += 16.0 * s->dims * s->np;                               // up and down link integral (or an up factor) per axis
