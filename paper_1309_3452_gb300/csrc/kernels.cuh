@@ -46,6 +46,7 @@ struct HalfStepArgs {
   HalfFields<P> h;
   FieldDesc f;
   int general;              // per-site FP64 field paths needed
+  int early;                // at most a block per SM (set by the launcher)
 };
 
 template <class P, int DIMS>

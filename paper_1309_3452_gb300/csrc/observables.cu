@@ -609,7 +609,8 @@ double measure_fp64_fma_tflops() {
 int observables_blocks(const int N[3], int dims) {
   const long long items = (long long)((N[0] + 31) / 32) * N[1] * (dims == 3 ? N[2] : 1);
   const long long b = (items + 7) / 8;
-  return (int)(b < 152 * 4 ? b : 152 * 4);
+  const int most = 4 * fused::sm_count();
+  return (int)(b < most ? b : most);
 }
 
 template <class P, int DIMS, bool kQuads, int kLink, bool kDens>

@@ -22,14 +22,14 @@ namespace {
 // there is room, not where there is work left: with a few blocks per SM some SMs
 // then get more than their share (67 x 39 x 24 Klein step, FP64, 720 blocks: 58 us
 // per step, 37 so; 96^3 249 and 64^2 5.0 either way).
-__device__ __forceinline__ void depends_half_step() {
+__device__ __forceinline__ void depends_half_step(bool early) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (gridDim.x * gridDim.y * gridDim.z <= 152u) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <class P, int DIMS, bool UPPER, int COEF, int LINK>
 __global__ void __launch_bounds__(128) half_step_kernel(const HalfStepArgs<P> a) {
-  depends_half_step();
+  depends_half_step(a.early != 0);
   using C = typename P::cplx;
   const int x = blockIdx.x * 32 + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -67,13 +67,14 @@ __global__ void __launch_bounds__(128) half_step_kernel(const HalfStepArgs<P> a)
 }
 
 template <class P, int DIMS, bool UPPER>
-void launch_one(const HalfStepArgs<P>& a, cudaStream_t s) {
+void launch_one(HalfStepArgs<P> a, cudaStream_t s) {
   // blocks of four rows, or of one where that leaves SMs without work (the FP64
   // pipe is narrow: 64^2 in 32 blocks kept 32 of 152 busy, 5.55 us per step; 4.97 in 128)
   const long long blocks4 = (long long)((a.N[0] + 31) / 32) * ((a.N[1] + 3) / 4) * (DIMS == 3 ? a.N[2] : 1);
   const int rows = blocks4 < 2 * fused::sm_count() ? 1 : 4;
   dim3 block(32, rows);
   dim3 grid((a.N[0] + 31) / 32, (a.N[1] + rows - 1) / rows, DIMS == 3 ? a.N[2] : 1);
+  a.early = (long long)grid.x * grid.y * grid.z <= fused::sm_count();
   const int c = a.h.coef_mode, l = a.h.link_mode;
   constexpr bool f32 = sizeof(typename P::real) == 4;
 #define HALF_STEP(COEF, LINK) launch_dependent(half_step_kernel<P, DIMS, UPPER, COEF, LINK>, grid, block, 0, s, a)

@@ -53,3 +53,8 @@ def test_no_copies_on_the_legacy_stream():
     """Kernels on a non-blocking stream are not ordered after what goes through the legacy one."""
     for name in sorted(os.listdir(CSRC)):
         assert not re.search(r"\bcuda(Memcpy|Memset)\(", source(name)), name
+
+
+def test_grid_rules_ask_for_the_device_size():
+    assert "152" not in source("step_split.cu")
+    assert "sm_count()" in body(source("observables.cu"), "int observables_blocks(")
