@@ -395,10 +395,6 @@ static HalfFields<P> half_fields(const dirac_sim* s, bool upper, double t) {
   return h;
 }
 
-static bool general_fields(const dirac_sim* s) {
-  return s->coef_mode == COEF_GENERAL || s->link_mode == LINK_GENERAL;
-}
-
 template <class P>
 static HalfStepArgs<P> half_args(dirac_sim* s, bool upper, double t) {
   HalfStepArgs<P> a;
@@ -412,7 +408,6 @@ static HalfStepArgs<P> half_args(dirac_sim* s, bool upper, double t) {
   a.rz = make_ratio<P>((s->dt / s->dx[2]) / rx);
   a.h = half_fields<P>(s, upper, t);
   a.f = field_desc(s);
-  a.general = general_fields(s);
   return a;
 }
 

@@ -96,13 +96,6 @@ __device__ __forceinline__ void row2d(const FusedArgs<P>& a, bool iso, int hx, i
   }
 }
 
-// the functional's terms of one (2+1)D row: new u1 and v of the row
-__device__ __forceinline__ void row_terms(float2 u1, const Quad& V, const Quad& S, double& e_n, double& e_c) {
-  e_n += (n2(u1) + n2(qlane(V, 0))) + n2(qlane(V, 1));
-  e_c += fmaf(V.re.y, S.re.y, fmaf(V.im.y, S.im.y, fmaf(V.re.x, S.re.x, V.im.x * S.im.x)));
-}
-
-
 // One work item (one strip over one chunk of rows) of one simulation, processed
 // by one warp: kT time steps of the chunk's rows.
 // kStepSlots: a Klein step's coefficients lie between the rows and the wave's factors

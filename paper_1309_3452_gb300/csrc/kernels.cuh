@@ -45,7 +45,6 @@ struct HalfStepArgs {
   typename P::Ratio ry, rz; // r_y/r_x, r_z/r_x
   HalfFields<P> h;
   FieldDesc f;
-  int general;              // per-site FP64 field paths needed
   int early;                // at most a block per SM (set by the launcher)
 };
 
@@ -104,12 +103,10 @@ struct BatchArgs {
   int nsims;
   int workers;                   // set by the launcher
 };
-// levels per work item and number of items the fused kernels use for a grid
-// (a FusedArgs chunk of 0 makes the launchers take fused_chunk's rule), with
-// `steps` time steps per pass (1; (2+1)D: 1 or 2)
-int fused_chunk(int dims, const int N[3], int steps);
-// the same for n grids in one batched launch (N[i] the extents): every chunk[i]
-// that is 0 is set
+// (`steps`: time steps per pass, 1; (2+1)D: 1 or 2)
+// levels per work item for n grids in one batched launch (N[i] the extents):
+// every chunk[i] that is 0 is set (launches of one grid take the rule for
+// themselves where FusedArgs's chunk is 0)
 void fused_batch_chunks(int dims, const int* const* N, int n, int steps, int* chunk);
 // chunk lengths worth timing, best first by the planner's model; returns the count
 int fused_candidates(int dims, const int N[3], int steps, int* out, int max);

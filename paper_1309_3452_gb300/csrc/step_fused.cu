@@ -153,8 +153,6 @@ ChunkShape shape_of(int dims, const int N[3], int steps) { return dims == 3 ? sh
 
 int launch_fused2d_two(const FusedArgs<F32>& a, cudaStream_t s) { return dispatch<2, 2>(a, s); }
 
-int fused_chunk(int dims, const int N[3], int steps) { return plan_chunk(shape_of(dims, N, steps)); }
-
 int fused_candidates(int dims, const int N[3], int steps, int* out, int max) {
   const ChunkShape g = shape_of(dims, N, steps);
   return rank_chunks(g.tiles, g.levels, g.workers, g.min_chunk, g.restart, out, max);
