@@ -1157,7 +1157,7 @@ static dirac_status steps_split(dirac_sim* s, long n, cudaStream_t st) {
 static bool per_site_path(const dirac_sim* s) {
   const int c = s->coef_mode, l = s->link_mode;
   if (c == COEF_GENERAL || l == LINK_GENERAL) return true;
-  if (c == COEF_SOFTCORE || c == COEF_SOFTCORR) return l == LINK_CONST || l == LINK_TABLE;
+  if (c == COEF_SOFTCORE || c == COEF_SOFTCORR) return l == LINK_CONST || (l == LINK_TABLE && c == COEF_SOFTCORR);
   return c == COEF_TABLE && l == LINK_CONST;
 }
 

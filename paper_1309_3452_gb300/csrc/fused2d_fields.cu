@@ -14,6 +14,7 @@ ALL_2D(COEF_UNIFORM, LINK_TABLE)
 ALL_2D(COEF_STEP, LINK_TABLE)
 ALL_2D(COEF_STEP_X, LINK_TABLE)
 ALL_2D(COEF_TABLE, LINK_TABLE)
+ALL_2D(COEF_SOFTCORE, LINK_TABLE)
 STEPS_2D(kAnyMode, kAnyMode, 1)
 
 }  // namespace fused

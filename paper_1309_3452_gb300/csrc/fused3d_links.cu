@@ -10,6 +10,7 @@ STEP_3D(COEF_STEP, LINK_CONST)
 STEP_3D(COEF_UNIFORM, LINK_TABLE)
 STEP_3D(COEF_STEP, LINK_TABLE)
 STEP_3D(COEF_TABLE, LINK_TABLE)
+STEP_3D(COEF_SOFTCORE, LINK_TABLE)
 
 }  // namespace fused
 }  // namespace dirac

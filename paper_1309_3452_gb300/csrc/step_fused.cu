@@ -105,6 +105,9 @@ int dispatch(const FusedArgs<F32>& a, cudaStream_t s) {
   if (c == COEF_SOFTCORE) {
     if (l == LINK_NONE) RUN(COEF_SOFTCORE, LINK_NONE);
     if (l == LINK_PLANE) RUN(COEF_SOFTCORE, LINK_PLANE);
+    // (the run-time path takes one value at a time and each loads the pair's link
+    // record: 96^3 574 us per step, 224 so; 512^2 42 and 22.5)
+    if (l == LINK_TABLE) RUN(COEF_SOFTCORE, LINK_TABLE);
     RUN(kAnyMode, kAnyMode);
   }
   if (c == COEF_SOFTCORR) {
