@@ -127,7 +127,9 @@ typedef enum {
  * per-value data.  Any other A that does not change in time (Apw_omega = 0
  * or Apw_amp = 0; Alink_omega = 0 or Alink_amp = 0) has its factors
  * exp(-i phi) tabulated once per simulation for DIRAC_FP32 (FP64 phases,
- * hi + lo float pairs); otherwise they are evaluated per site in FP64.
+ * hi + lo float pairs), and for DIRAC_FP64 where Apw_amp = 0 (the links
+ * towards +x, +y, +z, whose integrals they replace); otherwise they are
+ * evaluated per site in FP64.
  * dirac_norm_noalloc does not take A_links.  The upper
  * half-step uses the fields at time t, the lower half-step at t + dt/2 (the
  * time sheets of Eqs. ss1-ss4).
@@ -349,8 +351,9 @@ dirac_status dirac_check(dirac_sim* sim, double tol, dirac_check_report* out);
 
 /* Algorithmic HBM bytes of one site update (one cell advanced one full time
    step) on this simulation's path: every value read and written once, plus
-   a per-site coefficient (16 bytes) or static potential (8 bytes) read per
-   value where the potential needs one, and the vector potential's per-value
+   a per-site coefficient (16 bytes; absorbing layers are counted so too,
+   although the fused kernels' cells share most of theirs) or static
+   potential (8 bytes) read per value where the potential needs one, and the vector potential's per-value
    link data where it has some: two tabulated link factors (32 bytes) per axis
    and value, or two link integrals (16 bytes) per axis and value on the
    per-site path.  The roofline numerator of a time step.  0 for NULL. */

@@ -1,10 +1,12 @@
 // Shared device definitions of libdirac: precision traits, the staggered grid
 // geometry and the per-value update of the leap-frog scheme (arXiv:1309.3452).
 //
-// Device layout: one array per plane (A0,A1,B0,B1,C0,C1,D0,D1 in (3+1)D;
-// u0,u1,v0,v1 in (2+1)D), each [z][y][x] with x fastest, complex values
-// interleaved (float2 / double2).  Plane k starts at base + k*pstride
-// elements; pstride is a multiple of 64 elements.
+// Device layout (FP64, and FP32 with the plain half-step kernels): one array per
+// plane (A0,A1,B0,B1,C0,C1,D0,D1 in (3+1)D; u0,u1,v0,v1 in (2+1)D), each
+// [z][y][x] with x fastest, complex values interleaved (float2 / double2).
+// Plane k starts at base + k*pstride elements; pstride is a multiple of 64
+// elements.  The fused FP32 kernels hold both planes of a component together
+// (quad.cuh).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -285,7 +287,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // per step, now 112).  (The fused FP32
 // kernels keep both links of every value: with up links alone their tiles, each
 // at a level of its own, spread the reuse over more than L2, 128^3 538 us per
-// step against 380, and 565 with the next level prefetched to L2.)  GENERAL: per-site FP64.  COEF_SOFTCORE (FP32 kernels): a soft-core
+// step against 395, and 565 with the next level prefetched to L2.)  GENERAL: per-site FP64.  COEF_SOFTCORE (FP32 kernels): a soft-core
 // potential (with V0 and a Klein step, real) whose b is computed per value
 // in compensated FP32 from |x - c|^2 + a^2, itself summed from three small
 // per-axis tables of (X dx_a/2 - c_a)^2 (no per-site data).

@@ -37,8 +37,8 @@
 // in the long chains) and the barriers.  Tiles of 34 x 28 and 34 x 30 cells are
 // the largest that one block per SM can hold two cells per thread of: smaller
 // ones spend more on halo cells (14 rows: 6114 us per 512^3 laser step against
-// 3931).  us per step, with (re, im) lanes per value / now: 128^3 free 59.6 / 54.4, 203 x 149 x
-// 91 Klein step anisotropic 102 / 82.8, 512^3 laser 4879 / 3945, 160^3 layers
+// 3940).  us per step, with (re, im) lanes per value / now: 128^3 free 59.6 / 54.4, 203 x 149 x
+// 91 Klein step anisotropic 102 / 82.8, 512^3 laser 4879 / 3940, 160^3 layers
 // 227 / 141, 128^3 static links 670 / 395.
 //
 // Cells outside the grid (ragged last tiles) are wrapped periodically, so
@@ -101,15 +101,16 @@ struct LevelLoad {
 };
 
 // Thread geometry inside the (3+1)D tile (two cells per thread, rows ly and
-// ly + 1).  Warps 0..13 hold the columns 1..32 (lane -> x) of the row pairs
-// (0,1), (2,3), .., (26,27); rows 0 and 27 are halo rows, so warp 0's lower
-// cell and warp 13's upper cell are halo cells.  Warp 14 holds the halo
-// columns 0 and 33 of every row pair (28 threads) and four spare threads
-// (rows 28, 29 of shared memory, never stored).  Halo cells take part in the
-// upper half-step only, whose values the interior needs.
+// ly + 1).  Warp w < kPairs holds the columns 1..32 (lane -> x) of the row pair
+// (2w, 2w + 1); the first and the last row are halo rows, so warp 0's lower cell
+// and the last pair's upper cell are halo cells.  The last warp holds the
+// halo columns 0 and 33 of every row pair (2 kPairs threads) and the spare
+// threads that are left (four with 14 pairs, two with 15; rows of their own in shared
+// memory, never stored).  Halo cells take part in the upper half-step only,
+// whose values the interior needs.
 struct Thread3d {
   int slot;                // the lower cell's shared-memory slot, (ly + 1) * TW + lx (upper: slot + TW)
-  int lx, ly;              // position of the lower cell in the 34 x 28 tile
+  int lx, ly;              // position of the lower cell in the tile
   bool halo;               // warp-uniform: halo columns and spares (upper half-step only)
   bool h0, h1;             // warp-uniform: the lower / upper cell is a halo cell
 };
@@ -525,7 +526,7 @@ int workers3d() {
 // Row pairs of a grid's tiles: the fewer rows computed (tiles along y times
 // their rows, halo and ragged last tile included); 15 pairs at equal rows are 5 %
 // faster with a soft core (its arithmetic fills the four schedulers evenly; 512^3 laser
-// 3931 us per step against 4084 with 14 pairs, 570 rows against 560) and even
+// 3940 us per step against 4084 with 14 pairs, 570 rows against 560) and even
 // otherwise (160^3 layers with a coefficient record per cell 189 us per step with
 // 15 pairs, 180 rows, against 206 with 14, 196 rows; 128^3 free 57.7 against 54.2, 150 rows against 140).
 template <int COEF>

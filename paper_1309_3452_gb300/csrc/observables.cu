@@ -137,7 +137,9 @@ __device__ __forceinline__ Pair<P> load_pair(const ObsArgs<P>& a, int comp, long
 // us at 128^3 free / 4096^2 / 512^3 laser: with a block per 32 x 8 cells and z
 // range, a sincos per link, FP64 sums per cell and up to 65536 partials summed
 // by one warp 203 / 1449 / 79120; with this grid, link tables and FP64 sums
-// 55 / 215 / 9840; now 48 / 159 / 3945.
+// 55 / 215 / 9840; with the sums' errors in one float and rotations rounded before
+// their difference (fewer bits than the FP64 sums and rotations) 39 / 150 / 3890;
+// now, the kernel alone, 43 / 135 / 3950 (128^3 static links 167 and 210).
 template <class P, int DIMS, bool kQuads, int kLink, bool kDens>
 __global__ void __launch_bounds__(256) observables_kernel(const ObsArgs<P> a) {
   using C = typename P::cplx;
