@@ -11,9 +11,9 @@ namespace dirac {
 // dependents: the next kernel's blocks are placed while the last blocks of the
 // one before still run, and wait in depends() until that one has finished and
 // its writes are visible.  Every kernel launched this way calls depends() before
-// it touches memory, and reads what an earlier launch of its kind wrote by ordinary
-// loads (the wait orders those, not the read-only path), so the order of all work is that of plain launches; what
-// is saved is the launch latency between short kernels.
+// it touches memory, and reads what an earlier launch wrote by ordinary loads
+// (the wait orders those, not the read-only path), so the order of all work is
+// that of plain launches; what is saved is the launch latency between short kernels.
 // us per step, before and after: 96^3 FP64 254 / 249, 64^2 FP64 5.5 / 5.0,
 // 203x149x91 84.5 / 82.8, 300 x 260 3.16 / 3.09; long kernels unchanged.
 __device__ __forceinline__ void depends() {

@@ -131,8 +131,9 @@ __device__ __forceinline__ Pair<P> load_pair(const ObsArgs<P>& a, int comp, long
 // precision (FP32 states: products of two stored floats) and accumulated per
 // thread (SumOf), then in FP64 per warp (shuffles), per block and over the
 // blocks, in a fixed order, so the result is deterministic for a given grid.
-// Plane-wave link factors c - i s come from a table.  kLink: LINK_TABLE is the quads' table of factors; any
-// other vector potential (LINK_GENERAL) evaluates its phases in FP64.
+// Plane-wave link factors c - i s come from a table.  kLink: LINK_TABLE is the
+// quads' table of factors; any other vector potential (LINK_GENERAL) evaluates
+// its phases in FP64.
 // Bound: loads (14 16-byte records per cell, about 5 from L2 or HBM).
 // us at 128^3 free / 4096^2 / 512^3 laser: with a block per 32 x 8 cells and z
 // range, a sincos per link, FP64 sums per cell and up to 65536 partials summed
@@ -437,9 +438,9 @@ __global__ void softcore_corr_kernel(unsigned* __restrict__ out, const HalfField
 }
 
 // q times the link integrals of every value in the state layout: the value's
-// own link towards +dx_a/2 (slot 2a; alone, dirs = 1: slot a) and the link from its neighbour at
-// -dx_a/2 to it (slot 2a+1), which that neighbour (partner plane, cell shifted
-// with the periodic wrap) carries as its own up link
+// own link towards +dx_a/2 (slot 2a; alone, dirs = 1: slot a) and the link from
+// its neighbour at -dx_a/2 to it (slot 2a+1), which that neighbour (partner
+// plane, cell shifted with the periodic wrap) carries as its own up link
 template <int DIMS>
 __global__ void link_integral_table_kernel(double* __restrict__ out, const double* __restrict__ raw, int N0,
                                            int N1, int N2, long long pstride, double q, int dirs) {
